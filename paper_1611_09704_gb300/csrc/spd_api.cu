@@ -60,6 +60,14 @@ int plane_vec_ok(const spd_plane *p) {
            ((size_t)p->row_stride * eb) % need == 0;
 }
 
+// Rows the search kernel may fetch by bulk copies, whose addresses must be
+// multiples of 16 bytes whatever the storage type.  (Tiles start at multiples
+// of 16 samples within a row.)
+int plane_bulk_ok(const spd_plane *p) {
+    return reinterpret_cast<uintptr_t>(p->data) % 16 == 0 &&
+           ((size_t)p->row_stride * elem_bytes(p->dtype)) % 16 == 0;
+}
+
 int64_t entries_of(const spd_plane *p, int scope) { return scope == SPD_MSD_PER_ROW ? p->n_dm : 1; }
 
 bool scope_ok(int scope) { return scope == SPD_MSD_GLOBAL || scope == SPD_MSD_PER_ROW; }
@@ -246,7 +254,7 @@ spd_status range_consts(const spd_plane *p, const RangeProg &prog, const spd_msd
     rd.mu_tab = c.mu_tab;
     rd.flags = c.flags;
     rd.tiles_per_row = 0;   // the tile geometry is set by run_launch
-    rd.vec_ok = plane_vec_ok(p);
+    rd.vec_ok = plane_bulk_ok(p);
     rd.per_row = scope == SPD_MSD_PER_ROW;
     rd.R = 0;
     rd.span = 0;
