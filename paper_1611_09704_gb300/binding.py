@@ -283,6 +283,10 @@ def _workspace(nbytes: int, device) -> torch.Tensor:
     return torch.empty(max(int(nbytes), 1), dtype=torch.uint8, device=device)
 
 
+def _nbytes(t: torch.Tensor) -> int:
+    return t.numel() * t.element_size()
+
+
 def entries(plane: Plane, scope: int) -> int:
     return plane.n_dm if scope == MSD_PER_ROW else 1
 
@@ -300,7 +304,7 @@ def msd(x, scope=MSD_GLOBAL, nmax_sigma=0, *, stream=None, out=None, workspace=N
         out = torch.empty(max(n, 1) * MSD_BYTES, dtype=torch.uint8, device=pl.data.device)
     wsb = lib.spd_msd_workspace_bytes(ctypes.byref(cp), scope, nmax_sigma)
     ws = workspace if workspace is not None else _workspace(wsb, pl.data.device)
-    _check(lib.spd_msd(ctypes.byref(cp), scope, nmax_sigma, _ptr(out), _ptr(ws), wsb,
+    _check(lib.spd_msd(ctypes.byref(cp), scope, nmax_sigma, _ptr(out), _ptr(ws), _nbytes(ws),
                        _stream(stream)), "spd_msd")
     return out
 
@@ -455,7 +459,7 @@ def detect(x, msd_dev, widths, threshold, capacity, sigma_mode=SIGMA_SQRTN, scop
     wsb = lib.spd_detect_workspace_bytes(ctypes.byref(cp), ctypes.byref(prm))
     ws = workspace if workspace is not None else _workspace(wsb, dev)
     _check(lib.spd_detect(ctypes.byref(cp), ctypes.byref(prm), _ptr(msd_dev), _ptr(out),
-                          int(capacity), _ptr(result), _ptr(ws), wsb, _stream(stream)),
+                          int(capacity), _ptr(result), _ptr(ws), _nbytes(ws), _stream(stream)),
            "spd_detect")
     del keep
     return out, result
@@ -489,8 +493,8 @@ def search(x, widths, threshold, capacity, sigma_mode=SIGMA_SQRTN, scope=MSD_GLO
     wsb = lib.spd_search_workspace_bytes(ctypes.byref(cp), ctypes.byref(prm))
     ws = workspace if workspace is not None else _workspace(wsb, dev)
     _check(lib.spd_search(ctypes.byref(cp), ctypes.byref(prm), _ptr(out), int(capacity),
-                          _ptr(result), _ptr(msd_out), _ptr(ws), wsb, _stream(stream)),
-           "spd_search")
+                          _ptr(result), _ptr(msd_out), _ptr(ws), _nbytes(ws),
+                          _stream(stream)), "spd_search")
     del keep
     return out, result, msd_out
 
@@ -632,7 +636,7 @@ def search_batched(specs, capacity, tuning=None, *, stream=None, out=None, resul
     ws = workspace if workspace is not None else _workspace(wsb, dev)
     _check(lib.spd_search_batched(rg.arr, len(rg.specs), ctypes.byref(t) if t else None,
                                   _ptr(out), int(capacity), _ptr(result), _ptr(msd_out),
-                                  _ptr(ws), wsb, _stream(stream)), "spd_search_batched")
+                                  _ptr(ws), _nbytes(ws), _stream(stream)), "spd_search_batched")
     return out, result, msd_out
 
 

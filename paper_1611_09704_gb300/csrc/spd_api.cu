@@ -200,6 +200,63 @@ DetLayout det_layout(int64_t entries, int n_eval) {
     return l;
 }
 
+// Screening (see spd_internal.cuh): tables per scope entry and the lists, in
+// one piece after everything else a call keeps in its workspace.  A caller
+// whose workspace holds all but this piece gets the search without a screen.
+struct ScreenLayout {
+    size_t tab_off, grp_off, ctl_off, tiles_off, units_off, total;
+    int64_t tile_cap, unit_cap;
+};
+
+// Most tiles of the search kernel (256 threads: at least 192 units of 16
+// starts per tile) on a plane.
+int64_t screen_tiles(int64_t n_dm, int64_t n_samp) {
+    const int64_t per = 16 * (kSearchThreads - 64);
+    return n_dm * ((n_samp + per - 1) / per);
+}
+
+// Lists of a launch over `tiles` tiles; the tables of one range of `entries`
+// scope entries and n_groups width groups follow per range (screen_tables).
+ScreenLayout screen_lists(int64_t tiles) {
+    ScreenLayout l;
+    memset(&l, 0, sizeof(l));
+    l.tile_cap = tiles;
+    l.unit_cap = 8 * tiles + 1024;
+    l.ctl_off = 0;
+    l.tiles_off = l.ctl_off + align_up(kScrSlots * sizeof(ScreenCtl));
+    l.units_off = l.tiles_off + align_up((size_t)l.tile_cap * sizeof(uint32_t));
+    l.total = l.units_off + align_up((size_t)l.unit_cap * sizeof(uint64_t));
+    return l;
+}
+
+size_t screen_tables(int64_t entries, int n_groups) {
+    return align_up((size_t)entries * kScrTab * sizeof(float)) +
+           align_up((size_t)entries * n_groups * sizeof(float2));
+}
+
+size_t screen_bytes(int64_t n_dm, int64_t n_samp, int64_t entries, int n_groups) {
+    return screen_lists(screen_tiles(n_dm, n_samp)).total + screen_tables(entries, n_groups);
+}
+
+// As used by a call over one plane.
+size_t plane_screen_bytes(const spd_plane *p, int scope, const RangeProg &prog) {
+    return screen_bytes(p->n_dm, p->n_samp, entries_of(p, scope), prog.n_groups);
+}
+
+// The lists at `base` (null: no screen).
+ScreenLists lists_at(char *base, int64_t tiles) {
+    ScreenLists s;
+    memset(&s, 0, sizeof(s));
+    if (!base) return s;
+    const ScreenLayout l = screen_lists(tiles);
+    s.ctl = reinterpret_cast<ScreenCtl *>(base + l.ctl_off);
+    s.tiles = reinterpret_cast<uint32_t *>(base + l.tiles_off);
+    s.units = reinterpret_cast<uint64_t *>(base + l.units_off);
+    s.tile_cap = l.tile_cap;
+    s.unit_cap = l.unit_cap;
+    return s;
+}
+
 spd_status check_ws(const void *ws, size_t have, size_t need) {
     if (need == 0) return SPD_OK;
     if (!ws) return SPD_ERR_NO_MEMORY;
@@ -225,10 +282,12 @@ int nmax_of(const spd_search_params *q) {
     return q->widths && q->n_widths > 0 ? q->widths[q->n_widths - 1] : 0;
 }
 
-// Constants kernel for one range: 1/sigma_w per entry and width, mean, flags.
-spd_status range_consts(const spd_plane *p, const RangeProg &prog, const spd_msd_stats *msd_dev,
-                        int scope, int sigma_mode, spd_result *result, void *ws,
-                        cudaStream_t st, RangeDesc &rd, int skip_w1 = 0) {
+// Arguments of the constants of one range: 1/sigma_w per entry and width, mean,
+// flags; with `tables` (screen_tables bytes) the screen's and the groups'
+// factors, and with `ctl` the screen's counters zeroed.
+ConstArgs const_args(const spd_plane *p, const RangeProg &prog, const spd_msd_stats *msd_dev,
+                     int scope, int sigma_mode, spd_result *result, void *ws, int skip_w1,
+                     char *tables, ScreenCtl *ctl) {
     const int64_t entries = entries_of(p, scope);
     const DetLayout L = det_layout(entries, prog.n_eval);
     char *base = static_cast<char *>(ws);
@@ -241,8 +300,17 @@ spd_status range_consts(const spd_plane *p, const RangeProg &prog, const spd_msd
     c.flags = reinterpret_cast<int32_t *>(base + L.flags_off);
     c.result = result;
     c.skip_w1 = skip_w1;
-    SPD_CK(launch_consts(c, prog, st));
+    c.scr_tab = reinterpret_cast<float *>(tables);
+    c.grp_tab = tables ? reinterpret_cast<float2 *>(
+                             tables + align_up((size_t)entries * kScrTab * sizeof(float)))
+                       : nullptr;
+    c.ctl = ctl;
+    return c;
+}
 
+// The search's view of one range.
+RangeDesc range_desc(const spd_plane *p, const RangeProg &prog, int scope, const ConstArgs &c) {
+    RangeDesc rd;
     memset(&rd, 0, sizeof(rd));
     rd.data = p->data;
     rd.n_dm = p->n_dm;
@@ -253,6 +321,8 @@ spd_status range_consts(const spd_plane *p, const RangeProg &prog, const spd_msd
     rd.inv_tab = c.inv_tab;
     rd.mu_tab = c.mu_tab;
     rd.flags = c.flags;
+    rd.scr_tab = c.scr_tab;
+    rd.grp_tab = c.grp_tab;
     rd.tiles_per_row = 0;   // the tile geometry is set by run_launch
     rd.vec_ok = plane_bulk_ok(p);
     rd.per_row = scope == SPD_MSD_PER_ROW;
@@ -262,6 +332,18 @@ spd_status range_consts(const spd_plane *p, const RangeProg &prog, const spd_msd
     rd.sample_base = 0;
     rd.sample_shift = 0;
     rd.prog = prog;
+    return rd;
+}
+
+// Constants kernel of one range, and the search's view of it.
+spd_status range_consts(const spd_plane *p, const RangeProg &prog, const spd_msd_stats *msd_dev,
+                        int scope, int sigma_mode, spd_result *result, void *ws,
+                        cudaStream_t st, RangeDesc &rd, int skip_w1 = 0,
+                        char *tables = nullptr, ScreenCtl *ctl = nullptr) {
+    const ConstArgs c =
+        const_args(p, prog, msd_dev, scope, sigma_mode, result, ws, skip_w1, tables, ctl);
+    SPD_CK(launch_consts(c, prog, st));
+    rd = range_desc(p, prog, scope, c);
     return SPD_OK;
 }
 
@@ -274,9 +356,16 @@ thread_local uint32_t g_extra_tx = 0;
 // candidates, or with snr_out the plane output (every group evaluated).
 // Tiles of 16 starts per unit, units = the threads (128 or 256, 0 = the
 // default; plane output 256) less the halo's blocks.
+//
+// With `lists` (the ranges carrying the screen's tables) the launch is two:
+// the screen, then the search kernel over the tiles it lists and the live
+// units of the rest.  Not with 128-thread tiles (the lists are sized for 256), nor
+// while the test aid makes the search kernel's copies run out: then every
+// tile is searched.
 spd_status run_launch(const RangeDesc *rd, int n, int dtype, spd_candidate *out, int64_t cap,
                       spd_result *result, float *snr_out, uint16_t *width_out,
-                      int64_t out_stride, int ctas_per_sm, cudaStream_t st, int threads = 0) {
+                      int64_t out_stride, int ctas_per_sm, cudaStream_t st, int threads = 0,
+                      const ScreenLists *lists = nullptr) {
     static thread_local Launch L;
     memset(&L, 0, sizeof(L));
     const int nt = !snr_out && (threads == 128 || threads == 256) ? threads : kSearchThreads;
@@ -333,7 +422,28 @@ spd_status run_launch(const RangeDesc *rd, int n, int dtype, spd_candidate *out,
     L.units = units;
     const size_t smem = search_smem_bytes(L.R, raw, max_eval, kmax, G);
     if (smem > 227 * 1024) return SPD_ERR_UNSUPPORTED;
-    SPD_CK(launch_search(L, dtype, G, max_eval > 64, smem, ctas_per_sm, nt, st));
+    const bool screen = lists && lists->ctl && !snr_out && nt == kSearchThreads && !g_extra_tx &&
+                        tiles <= lists->tile_cap && tiles < (int64_t)1 << 24;
+    size_t lsmem = smem;
+    if (screen && tiles > 0) {
+        SPD_CK(launch_screen(L, *lists, dtype, st));
+        L.tile_list = lists->tiles;
+        L.tile_count = &lists->ctl->dense;
+        L.unit_list = lists->units;
+        L.unit_count = &lists->ctl->live;
+        L.unit_cap = (uint32_t)lists->unit_cap;
+        // a half-warp per unit where the tiles' shared memory holds them all;
+        // at least one warp (an even number: whole warps take part)
+        int wmax = 0;
+        for (int i = 0; i < n; ++i) wmax = rd[i].prog.wmax > wmax ? rd[i].prog.wmax : wmax;
+        L.live_blocks = ((15 + wmax) >> 4) + 1;
+        const size_t words = (size_t)live_words(L.live_blocks, G) * sizeof(float);
+        L.live_halves = (int)(smem / words) & ~1;
+        if (L.live_halves > nt / 16) L.live_halves = nt / 16;
+        if (L.live_halves < 2) L.live_halves = 2;
+        if (lsmem < words * L.live_halves) lsmem = words * L.live_halves;
+    }
+    SPD_CK(launch_search(L, dtype, G, max_eval > 64, lsmem, ctas_per_sm, nt, st));
     return SPD_OK;
 }
 
@@ -341,11 +451,21 @@ spd_status run_launch(const RangeDesc *rd, int n, int dtype, spd_candidate *out,
 spd_status run_detect(const spd_plane *p, const RangeProg &prog, const spd_msd_stats *msd_dev,
                       int scope, int sigma_mode, float thr, spd_candidate *out, int64_t cap,
                       spd_result *result, float *snr_out, uint16_t *width_out,
-                      int64_t out_stride, void *ws, cudaStream_t st) {
+                      int64_t out_stride, void *ws, cudaStream_t st, char *scr = nullptr) {
     RangeDesc rd;
-    SPD_TRY(range_consts(p, prog, msd_dev, scope, sigma_mode, result, ws, st, rd));
+    const int64_t tiles = screen_tiles(p->n_dm, p->n_samp);
+    const ScreenLists lists = lists_at(scr, tiles);
+    SPD_TRY(range_consts(p, prog, msd_dev, scope, sigma_mode, result, ws, st, rd, 0,
+                         scr ? scr + screen_lists(tiles).total : nullptr, lists.ctl));
     rd.threshold = thr;
-    return run_launch(&rd, 1, p->dtype, out, cap, result, snr_out, width_out, out_stride, 0, st);
+    return run_launch(&rd, 1, p->dtype, out, cap, result, snr_out, width_out, out_stride, 0, st,
+                      0, &lists);
+}
+
+// The screen's piece of a workspace after `used` bytes, or null where the
+// workspace ends before it.
+char *screen_at(void *ws, size_t have, size_t used, size_t bytes) {
+    return have >= used && have - used >= bytes ? static_cast<char *>(ws) + used : nullptr;
 }
 
 }  // namespace
@@ -381,8 +501,16 @@ size_t spd_msd_workspace_bytes(const spd_plane *plane, int32_t scope, int32_t nm
     return msd_layout(plane, nmax_sigma).total;
 }
 
-spd_status spd_msd(const spd_plane *plane, int32_t scope, int32_t nmax_sigma,
-                   spd_msd_stats *out_dev, void *workspace, size_t workspace_bytes, void *stream) {
+}  // extern "C"
+
+namespace {
+
+// spd_msd; and for a call that goes on to search: the result word set to 0
+// (`zero`), and for the global scope the constants of its one entry (`consts`,
+// `prog`), both in the MSD's own launches.  (Not for an empty plane.)
+spd_status msd_run(const spd_plane *plane, int32_t scope, int32_t nmax_sigma,
+                   spd_msd_stats *out_dev, void *workspace, size_t workspace_bytes, void *stream,
+                   spd_result *zero, const ConstArgs *consts, const RangeProg *prog) {
     SPD_TRY(check_plane(plane));
     if (!scope_ok(scope) || !out_dev) return SPD_ERR_INVALID_ARG;
     if (nmax_sigma < 0 || nmax_sigma == 1 || nmax_sigma > SPD_MAX_WIDTH)
@@ -404,12 +532,16 @@ spd_status spd_msd(const spd_plane *plane, int32_t scope, int32_t nmax_sigma,
         a.units_per_row = L.upr;
         a.vec_ok = plane_vec_ok(plane);
         a.parts = parts;
+        a.arrived = merge_counter(scratch, kMergeScratch);
+        a.result = zero;
         SPD_CK(launch_msd_partial(a, plane->dtype, st));
     }
     if (scope == SPD_MSD_PER_ROW && plane->n_dm == 0) return SPD_OK;
+    const bool nmax = nmax_sigma >= 2 && !plane_empty(plane);
     SPD_CK(launch_msd_merge(parts, plane->n_dm, L.upr, plane->n_samp,
-                            scope == SPD_MSD_PER_ROW, scratch, kMergeScratch, out_dev, st));
-    if (nmax_sigma >= 2 && !plane_empty(plane)) {
+                            scope == SPD_MSD_PER_ROW, scratch, kMergeScratch, out_dev,
+                            nmax ? nullptr : consts, prog, st));
+    if (nmax) {
         // sigma_Nmax of Eq. 5, centred on the mean just merged
         NmaxArgs n;
         n.data = plane->data;
@@ -425,9 +557,37 @@ spd_status spd_msd(const spd_plane *plane, int32_t scope, int32_t nmax_sigma,
         n.nb = nmax_blocks(nmax_sigma);
         n.tiles_per_row = L.ntpr;
         n.parts = reinterpret_cast<MsdPart *>(base + L.nmax_off);
-        SPD_CK(launch_nmax(n, plane->dtype, scratch, kMergeScratch, out_dev, st));
+        SPD_CK(launch_nmax(n, plane->dtype, scratch, kMergeScratch, out_dev, consts, prog, st));
     }
     return SPD_OK;
+}
+
+// The MSD of a range (not empty), its constants -- in the MSD's last launch
+// for the global scope -- and the search's view of it; with `zero` the result
+// word is set to 0 first.
+spd_status msd_and_consts(const spd_plane *p, const RangeProg &prog, const spd_search_params *q,
+                          spd_msd_stats *msd, void *msd_ws, size_t msd_bytes, spd_result *result,
+                          bool zero, void *det_ws, void *stream, RangeDesc &rd, int skip_w1,
+                          char *tables, ScreenCtl *ctl) {
+    const ConstArgs c = const_args(p, prog, msd, q->msd_scope, q->sigma_mode, result, det_ws,
+                                   skip_w1, tables, ctl);
+    const bool one = q->msd_scope == SPD_MSD_GLOBAL;
+    SPD_TRY(msd_run(p, q->msd_scope, nmax_of(q), msd, msd_ws, msd_bytes, stream,
+                    zero ? result : nullptr, one ? &c : nullptr, &prog));
+    if (!one) SPD_CK(launch_consts(c, prog, static_cast<cudaStream_t>(stream)));
+    rd = range_desc(p, prog, q->msd_scope, c);
+    rd.threshold = q->threshold;
+    return SPD_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
+spd_status spd_msd(const spd_plane *plane, int32_t scope, int32_t nmax_sigma,
+                   spd_msd_stats *out_dev, void *workspace, size_t workspace_bytes, void *stream) {
+    return msd_run(plane, scope, nmax_sigma, out_dev, workspace, workspace_bytes, stream, nullptr,
+                   nullptr, nullptr);
 }
 
 spd_status spd_msd_shard_partial(const spd_plane *plane, spd_msd_part *part_dev, void *workspace,
@@ -455,6 +615,8 @@ spd_status spd_msd_shard_partial(const spd_plane *plane, spd_msd_part *part_dev,
     a.units_per_row = L.upr;
     a.vec_ok = plane_vec_ok(plane);
     a.parts = parts;
+    a.arrived = nullptr;
+    a.result = nullptr;
     SPD_CK(launch_msd_partial(a, plane->dtype, st));
     SPD_CK(launch_fold_parts(parts, plane->n_dm * L.upr, scratch, kMergeScratch, out, st));
     return SPD_OK;
@@ -596,8 +758,10 @@ spd_status spd_cluster_rows(const float *snr, const uint16_t *width, int64_t n_d
 size_t spd_detect_workspace_bytes(const spd_plane *plane, const spd_search_params *params) {
     if (check_plane(plane) != SPD_OK || check_params(params) != SPD_OK) return 0;
     RangeProg prog;
-    if (compile_program(params->widths, params->n_widths, prog) != SPD_OK) return 0;
-    return det_layout(entries_of(plane, params->msd_scope), prog.n_eval).total;
+    if (compile_program(params->widths, params->n_widths, prog, 1, true) != SPD_OK) return 0;
+    const int64_t entries = entries_of(plane, params->msd_scope);
+    return det_layout(entries, prog.n_eval).total +
+           plane_screen_bytes(plane, params->msd_scope, prog);
 }
 
 spd_status spd_detect(const spd_plane *plane, const spd_search_params *params,
@@ -621,16 +785,19 @@ spd_status spd_detect(const spd_plane *plane, const spd_search_params *params,
     SPD_CK(cudaMemsetAsync(result_dev, 0, sizeof(spd_result), st));
     return run_detect(plane, prog, msd_dev, params->msd_scope, params->sigma_mode,
                       params->threshold, out, capacity, result_dev, nullptr, nullptr, 0,
-                      workspace, st);
+                      workspace, st,
+                      screen_at(workspace, workspace_bytes, need,
+                                plane_screen_bytes(plane, params->msd_scope, prog)));
 }
 
 size_t spd_search_workspace_bytes(const spd_plane *plane, const spd_search_params *params) {
     if (check_plane(plane) != SPD_OK || check_params(params) != SPD_OK) return 0;
     RangeProg prog;
-    if (compile_program(params->widths, params->n_widths, prog) != SPD_OK) return 0;
+    if (compile_program(params->widths, params->n_widths, prog, 1, true) != SPD_OK) return 0;
     const int64_t entries = entries_of(plane, params->msd_scope);
     return msd_layout(plane, nmax_of(params)).total +
-           align_up((size_t)entries * sizeof(spd_msd_stats)) + det_layout(entries, prog.n_eval).total;
+           align_up((size_t)entries * sizeof(spd_msd_stats)) +
+           det_layout(entries, prog.n_eval).total + plane_screen_bytes(plane, params->msd_scope, prog);
 }
 
 spd_status spd_search(const spd_plane *plane, const spd_search_params *params,
@@ -655,11 +822,16 @@ spd_status spd_search(const spd_plane *plane, const spd_search_params *params,
     SPD_TRY(check_ws(workspace, workspace_bytes, need));
     char *base = static_cast<char *>(workspace);
     spd_msd_stats *msd = msd_out_dev ? msd_out_dev : reinterpret_cast<spd_msd_stats *>(base + ML.total);
-    SPD_TRY(spd_msd(plane, params->msd_scope, nmax_of(params), msd, base, ML.total, stream));
-    SPD_CK(cudaMemsetAsync(result_dev, 0, sizeof(spd_result), st));
-    return run_detect(plane, prog, msd, params->msd_scope, params->sigma_mode,
-                      params->threshold, out, capacity, result_dev, nullptr, nullptr, 0,
-                      base + ML.total + msd_bytes, st);
+    char *scr = screen_at(workspace, workspace_bytes, need,
+                          plane_screen_bytes(plane, params->msd_scope, prog));
+    const int64_t tiles = screen_tiles(plane->n_dm, plane->n_samp);
+    const ScreenLists lists = lists_at(scr, tiles);
+    RangeDesc rd;
+    SPD_TRY(msd_and_consts(plane, prog, params, msd, base, ML.total, result_dev, true,
+                           base + ML.total + msd_bytes, stream, rd, 0,
+                           scr ? scr + screen_lists(tiles).total : nullptr, lists.ctl));
+    return run_launch(&rd, 1, plane->dtype, out, capacity, result_dev, nullptr, nullptr, 0, 0, st,
+                      0, &lists);
 }
 
 }  // extern "C"
@@ -669,6 +841,9 @@ namespace {
 struct BatchLayout {
     size_t msd_off[kMaxRanges], stats_off[kMaxRanges], det_off[kMaxRanges], total;
     size_t msd_bytes[kMaxRanges];
+    // after these, the screen's piece: the lists, then each range's tables
+    int64_t scr_tiles;
+    size_t scr_tab_off[kMaxRanges], scr_bytes;
 };
 
 spd_status batch_plan(const spd_range *ranges, int n, const spd_tuning *tuning,
@@ -696,6 +871,14 @@ spd_status batch_plan(const spd_range *ranges, int n, const spd_tuning *tuning,
         off += align_up(det_layout(entries, progs[i].n_eval).total);
     }
     L.total = off;
+    L.scr_tiles = 0;
+    for (int i = 0; i < n; ++i) L.scr_tiles += screen_tiles(ranges[i].plane.n_dm, ranges[i].plane.n_samp);
+    L.scr_bytes = screen_lists(L.scr_tiles).total;
+    for (int i = 0; i < n; ++i) {
+        L.scr_tab_off[i] = L.scr_bytes;
+        L.scr_bytes += screen_tables(entries_of(&ranges[i].plane, ranges[i].params.msd_scope),
+                                     progs[i].n_groups);
+    }
     return SPD_OK;
 }
 
@@ -713,7 +896,7 @@ size_t spd_search_batched_workspace_bytes(const spd_range *ranges, int32_t n_ran
     RangeProg progs[kMaxRanges];
     BatchLayout L;
     if (batch_plan(ranges, n_ranges, tuning, progs, L) != SPD_OK) return 0;
-    return L.total;
+    return L.total + L.scr_bytes;
 }
 
 spd_status spd_search_batched(const spd_range *ranges, int32_t n_ranges,
@@ -742,7 +925,9 @@ spd_status batched_impl(const spd_range *ranges, int32_t n_ranges, const spd_tun
     SPD_TRY(check_ws(workspace, workspace_bytes, L.total));
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     char *base = static_cast<char *>(workspace);
-    SPD_CK(cudaMemsetAsync(result_dev, 0, sizeof(spd_result), st));
+
+    char *scr = screen_at(workspace, workspace_bytes, L.total, L.scr_bytes);
+    const ScreenLists lists = lists_at(scr, L.scr_tiles);
 
     // (a) per range, and the constants of (c)
     RangeDesc rds[kMaxRanges];
@@ -755,20 +940,22 @@ spd_status batched_impl(const spd_range *ranges, int32_t n_ranges, const spd_tun
                                          : reinterpret_cast<spd_msd_stats *>(base + L.stats_off[i]);
         msd_pos += entries;
         if (plane_empty(&r.plane)) continue;
-        SPD_TRY(spd_msd(&r.plane, r.params.msd_scope, nmax_of(&r.params), msd,
-                        base + L.msd_off[i], L.msd_bytes[i], stream));
         // a decimated level evaluates only its listed widths
         const int skip_w1 = shifts && shifts[i] > 0 && r.params.widths[0] != 1;
-        SPD_TRY(range_consts(&r.plane, progs[i], msd, r.params.msd_scope, r.params.sigma_mode,
-                             result_dev, base + L.det_off[i], st, rds[i], skip_w1));
-        rds[i].threshold = r.params.threshold;
+        // the first range's MSD sets the result word to 0
+        SPD_TRY(msd_and_consts(&r.plane, progs[i], &r.params, msd, base + L.msd_off[i],
+                               L.msd_bytes[i], result_dev, n_live == 0, base + L.det_off[i],
+                               stream, rds[i], skip_w1, scr ? scr + L.scr_tab_off[i] : nullptr,
+                               lists.ctl));
         rds[i].dm_offset = r.dm_offset;
         rds[i].sample_shift = shifts ? shifts[i] : 0;
         live[n_live++] = i;
     }
+    if (!n_live) SPD_CK(cudaMemsetAsync(result_dev, 0, sizeof(spd_result), st));
     // (b, c, d): one persistent launch per class of ranges with equal G,
     // storage type and bulk-copy eligibility
     bool done[kMaxRanges] = {false};
+    int launches = 0;
     for (int a = 0; a < n_live; ++a) {
         const int i = live[a];
         if (done[i]) continue;
@@ -782,9 +969,10 @@ spd_status batched_impl(const spd_range *ranges, int32_t n_ranges, const spd_tun
             grp[m++] = rds[j];
             done[j] = true;
         }
+        const ScreenLists sl = lists.slot(launches++);
         SPD_TRY(run_launch(grp, m, ranges[i].plane.dtype, out, capacity, result_dev, nullptr,
                            nullptr, 0, tuning ? tuning->ctas_per_sm : 0, st,
-                           tuning ? tuning->tile_threads : 0));
+                           tuning ? tuning->tile_threads : 0, &sl));
     }
     return SPD_OK;
 }
@@ -796,7 +984,7 @@ struct DecLayout {
     int lmax;
     int64_t n[kMaxDecLevel + 1], stride[kMaxDecLevel + 1];
     size_t plane_off[kMaxDecLevel + 1];
-    size_t batch_off, batch_bytes, total;
+    size_t batch_off, total, scr_bytes;   // total: without the screen's piece
 };
 
 spd_status dec_plan(const spd_plane *plane, const spd_level *levels, int32_t n_levels,
@@ -852,8 +1040,8 @@ spd_status dec_plan(const spd_plane *plane, const spd_level *levels, int32_t n_l
     BatchLayout B;
     SPD_TRY(batch_plan(ranges, n_levels, nullptr, progs, B));
     D.batch_off = off;
-    D.batch_bytes = B.total;
     D.total = off + align_up(B.total);
+    D.scr_bytes = B.scr_bytes;
     return SPD_OK;
 }
 
@@ -867,7 +1055,7 @@ size_t spd_search_decimated_workspace_bytes(const spd_plane *plane, const spd_le
     int shifts[SPD_MAX_LEVELS];
     DecLayout D;
     if (dec_plan(plane, levels, n_levels, 1.f, ranges, shifts, D, nullptr) != SPD_OK) return 0;
-    return D.total;
+    return D.total + D.scr_bytes;
 }
 
 spd_status spd_search_decimated(const spd_plane *plane, const spd_level *levels, int32_t n_levels,
@@ -899,7 +1087,7 @@ spd_status spd_search_decimated(const spd_plane *plane, const spd_level *levels,
                                     D.stride[l], st));
     }
     return batched_impl(ranges, n_levels, nullptr, shifts, out, capacity, result_dev, msd_out_dev,
-                        base + D.batch_off, D.batch_bytes, stream);
+                        base + D.batch_off, workspace_bytes - D.batch_off, stream);
 }
 
 }  // extern "C"
@@ -936,6 +1124,7 @@ spd_status stream_layout(int64_t n_dm, int32_t dtype, const spd_search_params *p
 struct PushLayout {
     int64_t cstride;
     size_t comb_off, msd_off, msd_bytes, stats_off, det_off, total;
+    size_t scr_bytes;   // the screen's piece, after total
 };
 
 PushLayout push_layout(int64_t n_dm, int64_t max_chunk, int32_t dtype, const StreamLayout &S,
@@ -953,6 +1142,7 @@ PushLayout push_layout(int64_t n_dm, int64_t max_chunk, int32_t dtype, const Str
     L.stats_off = L.msd_off + align_up(L.msd_bytes);
     L.det_off = L.stats_off + align_up((size_t)S.entries * sizeof(spd_msd_stats));
     L.total = L.det_off + align_up(det_layout(S.entries, prog.n_eval).total);
+    L.scr_bytes = screen_bytes(n_dm, L.cstride, S.entries, prog.n_groups);
     return L;
 }
 
@@ -970,7 +1160,7 @@ spd_status stream_search(const spd_stream_info *info, const RangeProg &prog,
                          const spd_search_params *params, const void *comb, int64_t cstride,
                          int64_t n, int64_t n_emit, const float *scale, const float *offset,
                          const spd_msd_stats *stats, spd_candidate *out, int64_t cap,
-                         spd_result *result, void *det_ws, cudaStream_t st) {
+                         spd_result *result, void *det_ws, char *scr, cudaStream_t st) {
     spd_plane cp;
     memset(&cp, 0, sizeof(cp));
     cp.data = comb;
@@ -981,12 +1171,14 @@ spd_status stream_search(const spd_stream_info *info, const RangeProg &prog,
     cp.row_scale = scale;
     cp.row_offset = offset;
     RangeDesc rd;
+    const int64_t tiles = screen_tiles(info->n_dm, cstride);
+    const ScreenLists lists = lists_at(scr, tiles);
     SPD_TRY(range_consts(&cp, prog, stats, params->msd_scope, params->sigma_mode, result, det_ws,
-                         st, rd));
+                         st, rd, 0, scr ? scr + screen_lists(tiles).total : nullptr, lists.ctl));
     rd.threshold = params->threshold;
     rd.n_emit = n_emit;
     rd.sample_base = info->seen - info->halo;
-    return run_launch(&rd, 1, info->dtype, out, cap, result, nullptr, nullptr, 0, 0, st);
+    return run_launch(&rd, 1, info->dtype, out, cap, result, nullptr, nullptr, 0, 0, st, 0, &lists);
 }
 
 }  // namespace
@@ -1006,7 +1198,8 @@ size_t spd_stream_workspace_bytes(int64_t n_dm, int64_t max_chunk, int32_t dtype
     StreamLayout S;
     if (max_chunk < 0 || max_chunk > INT32_MAX) return 0;
     if (stream_layout(n_dm, dtype, params, prog, S) != SPD_OK) return 0;
-    return push_layout(n_dm, max_chunk, dtype, S, prog).total;
+    const PushLayout P = push_layout(n_dm, max_chunk, dtype, S, prog);
+    return P.total + P.scr_bytes;
 }
 
 spd_status spd_stream_reset(spd_stream_info *info, void *state_dev, int64_t n_dm, int32_t dtype,
@@ -1101,6 +1294,8 @@ spd_status spd_stream_push(spd_stream_info *info, void *state_dev, const spd_pla
     ma.vec_ok = plane_vec_ok(&in_place);
     MsdPart *parts = reinterpret_cast<MsdPart *>(ws + P.msd_off);
     ma.parts = parts;
+    ma.arrived = nullptr;
+    ma.result = nullptr;
     SPD_CK(launch_msd_partial(ma, chunk->dtype, st));
     spd_msd_stats *stats =
         msd_out_dev ? msd_out_dev : reinterpret_cast<spd_msd_stats *>(ws + P.stats_off);
@@ -1111,7 +1306,8 @@ spd_status spd_stream_push(spd_stream_info *info, void *state_dev, const spd_pla
     const int64_t hold = n < (int64_t)(prog.wmax - 1) ? n : (int64_t)(prog.wmax - 1);
     const int64_t n_emit = n - hold;
     SPD_TRY(stream_search(info, prog, params, comb, P.cstride, n, n_emit, chunk->row_scale,
-                          chunk->row_offset, stats, out, capacity, result_dev, ws + P.det_off, st));
+                          chunk->row_offset, stats, out, capacity, result_dev, ws + P.det_off,
+                          screen_at(workspace, workspace_bytes, P.total, P.scr_bytes), st));
     if (hold > 0)
         SPD_CK(cudaMemcpy2DAsync(halo, S.halo_cap * eb, comb + n_emit * eb, P.cstride * eb,
                                  hold * eb, info->n_dm, cudaMemcpyDeviceToDevice, st));
@@ -1169,7 +1365,8 @@ spd_status spd_stream_flush(spd_stream_info *info, void *state_dev,
                               ? reinterpret_cast<const float *>(state + S.offset_off)
                               : nullptr;
     SPD_TRY(stream_search(info, prog, params, ws + P.comb_off, P.cstride, H, H, scale, offset,
-                          stats, out, capacity, result_dev, ws + P.det_off, st));
+                          stats, out, capacity, result_dev, ws + P.det_off,
+                          screen_at(workspace, workspace_bytes, P.total, P.scr_bytes), st));
     info->halo = 0;
     return SPD_OK;
 }
@@ -1206,6 +1403,7 @@ struct HostLayout {
     int64_t dstride;
     size_t plane_off, scale_off, offset_off, search_off, msd_ws_bytes, result_off, msd_off,
         out_off, total;
+    size_t scr_bytes;   // the screen's piece, after total
 };
 
 spd_status host_layout(const spd_plane *hp, const spd_search_params *q, int64_t capacity,
@@ -1216,10 +1414,14 @@ spd_status host_layout(const spd_plane *hp, const spd_search_params *q, int64_t 
     spd_plane dp = *hp;
     dp.data = reinterpret_cast<void *>(256);   // any aligned address: sizes only
     dp.row_stride = H.dstride;
-    const size_t search_bytes = spd_search_workspace_bytes(&dp, q);
-    if (!search_bytes) return SPD_ERR_INVALID_ARG;
+    static thread_local RangeProg prog;
+    if (check_plane(&dp) != SPD_OK || check_params(q) != SPD_OK ||
+        compile_program(q->widths, q->n_widths, prog, 1, true) != SPD_OK)
+        return SPD_ERR_INVALID_ARG;
     H.msd_ws_bytes = msd_layout(&dp, nmax_of(q)).total;
     const int64_t entries = entries_of(hp, q->msd_scope);
+    const size_t search_bytes = H.msd_ws_bytes + align_up((size_t)entries * sizeof(spd_msd_stats)) +
+                                det_layout(entries, prog.n_eval).total;
     H.plane_off = 0;
     H.scale_off = align_up((size_t)hp->n_dm * H.dstride * eb);
     H.offset_off = H.scale_off + align_up((size_t)hp->n_dm * sizeof(float));
@@ -1228,6 +1430,7 @@ spd_status host_layout(const spd_plane *hp, const spd_search_params *q, int64_t 
     H.msd_off = H.result_off + kAlign;
     H.out_off = H.msd_off + align_up((size_t)entries * sizeof(spd_msd_stats));
     H.total = H.out_off + align_up((size_t)capacity * sizeof(spd_candidate));
+    H.scr_bytes = plane_screen_bytes(&dp, q->msd_scope, prog);
     return SPD_OK;
 }
 
@@ -1293,7 +1496,7 @@ size_t spd_search_host_workspace_bytes(const spd_plane *plane, const spd_search_
     if (check_plane(plane) != SPD_OK || check_params(params) != SPD_OK || capacity < 0) return 0;
     HostLayout H;
     if (host_layout(plane, params, capacity, H) != SPD_OK) return 0;
-    return H.total;
+    return H.total + H.scr_bytes;
 }
 
 spd_status spd_search_host(const spd_plane *host_plane, const spd_search_params *params,
@@ -1341,15 +1544,16 @@ spd_status spd_search_host(const spd_plane *host_plane, const spd_search_params 
         dp.row_offset = of;
     }
 
-    // (a) the MSD of the whole plane, the result word zeroed, then the
+    // (a) the result word set to 0, the MSD of the whole plane and the
     // constants of every row once
     char *sws = base + H.search_off;
-    SPD_TRY(spd_msd(&dp, params->msd_scope, nmax_of(params), msd, sws, H.msd_ws_bytes, stream));
-    SPD_CK(cudaMemsetAsync(res, 0, sizeof(spd_result), st));
     RangeDesc rd;
-    SPD_TRY(range_consts(&dp, prog, msd, params->msd_scope, params->sigma_mode, res,
-                         sws + H.msd_ws_bytes, st, rd));
-    rd.threshold = params->threshold;
+    char *scr = screen_at(workspace, workspace_bytes, H.total, H.scr_bytes);
+    const int64_t scr_tiles = screen_tiles(n_dm, host_plane->n_samp);
+    const ScreenLists lists = lists_at(scr, scr_tiles);
+    SPD_TRY(msd_and_consts(&dp, prog, params, msd, sws, H.msd_ws_bytes, res, true,
+                           sws + H.msd_ws_bytes, stream, rd, 0,
+                           scr ? scr + screen_lists(scr_tiles).total : nullptr, lists.ctl));
 
     // (b, c, d) by blocks of rows; block b's records go out while b + 1 runs
     HostAux *aux = nullptr;
@@ -1367,9 +1571,15 @@ spd_status spd_search_host(const spd_plane *host_plane, const spd_search_params 
             rb.inv_tab += r0 * prog.n_eval;
             rb.mu_tab += r0;
             rb.flags += r0;
+            if (scr) {
+                rb.scr_tab += r0 * kScrTab;
+                rb.grp_tab += r0 * prog.n_groups;
+            }
         }
         rb.dm_offset = (int32_t)r0;
-        SPD_TRY(run_launch(&rb, 1, dp.dtype, dev_out, capacity, res, nullptr, nullptr, 0, 0, st));
+        const ScreenLists sl = lists.slot(b);
+        SPD_TRY(run_launch(&rb, 1, dp.dtype, dev_out, capacity, res, nullptr, nullptr, 0, 0, st, 0,
+                           &sl));
         SPD_CK(cudaMemcpyAsync(aux->pin + b, res, sizeof(spd_result), cudaMemcpyDeviceToHost, st));
         SPD_CK(cudaEventRecord(aux->ev[b], st));
     }

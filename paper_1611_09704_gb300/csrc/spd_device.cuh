@@ -119,6 +119,49 @@ __device__ __forceinline__ void load4v<SPD_BF16>(const __nv_bfloat16 *p, float &
     a = lo.x; b = lo.y; c = hi.x; d = hi.y;
 }
 
+// ------------------------------------------------ positions of a window
+
+// Word of position p: 16 positions take kSPad words.
+__device__ __forceinline__ int sadr(int p) { return (p & 15) + kSPad * (p >> 4); }
+
+// Centred values y = (x - mu.hi) - mu.lo of window positions p .. p+N-1
+// (x = fmaf(scale, q, offset) for scaled storage), -inf at and past `have`.
+// Elements below nraw come from the raw staging buffer, the rest of the row
+// from global memory.
+template <int DT, int N>
+__device__ __forceinline__ void load_centred(float *v, const typename Elem<DT>::T *raw,
+                                             const typename Elem<DT>::T *gsrc, int p, int nraw,
+                                             int have, bool has_sc, float sc, float of, float2 mu) {
+    const float2 mh = make_float2(-mu.x, -mu.x), ml = make_float2(-mu.y, -mu.y);
+    if (p + N <= nraw) {
+#pragma unroll
+        for (int u = 0; u < N / 4; ++u) {
+            float a, b, c, d;
+            load4v<DT>(raw + p + 4 * u, a, b, c, d);
+            float2 x0 = make_float2(a, b), x1 = make_float2(c, d);
+            if (has_sc) {
+                const float2 s2 = make_float2(sc, sc), o2 = make_float2(of, of);
+                x0 = fma2(s2, x0, o2);
+                x1 = fma2(s2, x1, o2);
+            }
+            x0 = add2(add2(x0, mh), ml);
+            x1 = add2(add2(x1, mh), ml);
+            v[4 * u] = x0.x; v[4 * u + 1] = x0.y; v[4 * u + 2] = x1.x; v[4 * u + 3] = x1.y;
+        }
+    } else {
+#pragma unroll
+        for (int e = 0; e < N; ++e) {
+            const int q = p + e;
+            float x = 0.f;
+            if (q < nraw) x = Elem<DT>::cvt(raw[q]);
+            else if (q < have) x = Elem<DT>::cvt(gsrc[q]);
+            if (has_sc) x = fmaf(sc, x, of);
+            x = __fsub_rn(__fsub_rn(x, mu.x), mu.y);
+            v[e] = q < have ? x : -INFINITY;
+        }
+    }
+}
+
 // ------------------------------------------------------- double-float sums
 
 __device__ __forceinline__ float2 two_sum(float a, float b) {

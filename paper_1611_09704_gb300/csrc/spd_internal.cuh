@@ -50,7 +50,14 @@ struct MsdArgs {
     int64_t units_per_row;
     int vec_ok;          // 16-byte aligned rows: vector loads allowed
     MsdPart *parts;      // [n_dm * units_per_row]
+    unsigned *arrived;   // set to 0 (null: nothing), for the merge that follows
+    spd_result *result;  // set to 0 (null: nothing)
 };
+
+// The arrival counter of a merge: scratch's last place.
+inline unsigned *merge_counter(MsdPart *scratch, int n_scratch) {
+    return reinterpret_cast<unsigned *>(scratch + n_scratch - 1);
+}
 
 // Arguments of the sigma_Nmax pass (Eq. 5): tiles of 4096 starts per row.
 struct NmaxArgs {
@@ -111,6 +118,8 @@ struct RangeDesc {
     const float *inv_tab;       // [entries][n_eval]: 1 / sigma_w, FP32
     const float2 *mu_tab;       // [entries]: mean split into hi + lo FP32
     const int32_t *flags;       // [entries]: nonzero = degenerate sigma
+    const float *scr_tab;       // screening: see ConstArgs (null: not screened)
+    const float2 *grp_tab;
     int64_t tile0;              // first launch-wide tile index of this range
     int64_t tiles_per_row;
     int32_t vec_ok;             // 16-byte aligned rows: bulk (TMA) copies allowed
@@ -146,6 +155,12 @@ struct Launch {
     int32_t kmax;               // search kernel: levels of the block max table
     int32_t units;              // search kernel: units of 16 starts per tile (<= threads)
     int32_t chunk;              // search kernel: tiles per scheduling chunk (set at launch)
+    const uint32_t *tile_list;  // search kernel: the tiles to search (null: all n_tiles)
+    const uint32_t *tile_count; // and how many they are
+    const uint64_t *unit_list;  // then single units (null: none), tile << 8 | unit
+    const uint32_t *unit_count; // may exceed unit_cap, the list's room
+    uint32_t unit_cap;
+    int32_t live_blocks, live_halves;   // blocks and half-warps they are searched with
     RangeDesc rng[kMaxRanges];
 };
 
@@ -218,6 +233,56 @@ inline size_t search_smem_bytes(int RM, int raw_bytes, int max_eval, int kmax, i
     return search_smem(RM, raw_bytes, max_eval, kmax, G).total;
 }
 
+// ---------------------------------------------------------------- screening
+
+// The candidate search in three launches: a screen of the whole plane that
+// reads every sample once and keeps, per unit of 16 starts, only whether any
+// candidate can start there; the search kernel over the tiles with many such
+// live units; and one half-warp per live unit for the rest.
+//
+// The screen's bounds are per class of evaluated widths: widths 1..8, 9..16,
+// and (2^(c+2), 2^(c+3)] for c = 2 .. 9 (17..32 up to 2049..4096).
+constexpr int kScrClasses = 10;
+constexpr int kScrTab = 12;         // floats per scope entry: see ConstArgs::scr_tab
+constexpr int kScrSlots = 16;       // sets of counters: launches of one call
+// Live units of a tile beyond which the tile is searched whole.  A unit takes a
+// half-warp some 800 warp instructions, a tile the search kernel 15,000.
+constexpr int kScrDense = 16;
+
+__host__ __device__ inline int screen_class(int w) {
+    int c = w > 8 ? 1 : 0;
+    for (int h = 16; w > h; h *= 2) ++c;
+    return c;
+}
+
+// Counters of one screened launch, zeroed by the constants kernel.
+struct ScreenCtl {
+    uint32_t dense;       // tiles in the list of tiles
+    uint32_t live;        // units in the list of units (may exceed its capacity)
+    uint32_t reserved[2];
+};
+
+// Where a screened launch keeps its lists (null ctl: not screened).
+struct ScreenLists {
+    ScreenCtl *ctl;
+    uint32_t *tiles;      // launch-wide tile indexes, room for every tile
+    uint64_t *units;      // tile << 8 | unit of the tile
+    int64_t tile_cap, unit_cap;
+
+    // The same lists for launch k of a call: counters of its own.
+    ScreenLists slot(int k) const {
+        ScreenLists s = *this;
+        if (s.ctl) s.ctl += k;
+        return s;
+    }
+};
+
+// Shared words of one half-warp's live unit: y, P and (G > 1) S_G in kSPad
+// words per block, then per block its sum, largest prefix and energy prefix.
+__host__ __device__ inline int live_words(int blocks, int G) {
+    return (blocks * kSPad * (G > 1 ? 3 : 2) + 3 * blocks + 1 + 3) & ~3;   // 16-byte pieces
+}
+
 struct ConstArgs {
     const spd_msd_stats *msd;   // [entries]
     int entries;
@@ -225,6 +290,12 @@ struct ConstArgs {
     float *inv_tab;
     float2 *mu_tab;
     int32_t *flags;
+    // screening (null: not screened).  Per entry: the largest 1/sigma_w of
+    // each class, then the largest w / sigma_w^2 of class 0 and of classes 0
+    // and 1; per entry and group, the bounds' factors of the search kernel
+    float *scr_tab;             // [entries][kScrTab]
+    float2 *grp_tab;            // [entries][n_groups]
+    ScreenCtl *ctl;             // [kScrSlots], zeroed here
     spd_result *result;   // may be null: status set on a degenerate entry (count untouched)
     int skip_w1;          // eval index 0 (the width-1 start) takes no part: 1/sigma = NaN
 };
@@ -233,7 +304,10 @@ struct ConstArgs {
 cudaError_t launch_msd_partial(const MsdArgs &a, int dtype, cudaStream_t s);
 cudaError_t launch_msd_merge(const MsdPart *parts, int64_t n_dm, int64_t units_per_row,
                              int64_t n_samp, int per_row, MsdPart *scratch, int n_scratch,
-                             spd_msd_stats *out, cudaStream_t s);
+                             spd_msd_stats *out, const ConstArgs *consts, const RangeProg *prog,
+                             cudaStream_t s);
+// Global scope: with consts and prog the merge's launch forms the constants
+// too.  The partials' launch has set merge_counter(scratch, n_scratch) to 0.
 cudaError_t launch_consts(const ConstArgs &a, const RangeProg &prog, cudaStream_t s);
 cudaError_t launch_stream_msd(const MsdPart *parts, int64_t n_dm, int64_t upr, int per_row,
                               MsdPart *state, spd_msd_stats *out, cudaStream_t s);
@@ -249,12 +323,15 @@ cudaError_t launch_fold_parts(const MsdPart *parts, int64_t n_parts, MsdPart *sc
 cudaError_t launch_merge_shards(const MsdPart *parts, int n, int what, int nmax,
                                 spd_msd_stats *out, cudaStream_t s);
 cudaError_t launch_nmax(const NmaxArgs &a, int dtype, MsdPart *scratch, int n_scratch,
-                        spd_msd_stats *out, cudaStream_t s);
+                        spd_msd_stats *out, const ConstArgs *consts, const RangeProg *prog,
+                        cudaStream_t s);
 // The candidate search (search kernel): same launch description with the
 // ranges' tiles of 16 * threads starts (threads = 128 or 256), kmax set.
 cudaError_t launch_search(const Launch &L, int dtype, int G, bool multi_block, size_t smem,
                           int ctas_per_sm, int threads, cudaStream_t s);
 constexpr int kSearchThreads = 256;   // threads of a search CTA by default
+// The screen of a launch's ranges (geometry as for launch_search).
+cudaError_t launch_screen(const Launch &L, const ScreenLists &S, int dtype, cudaStream_t s);
 // x[2j] + x[2j+1] of a plane (dequantised) into an FP32 plane, j < n_out.
 cudaError_t launch_decimate2(const spd_plane &p, float *dst, int64_t n_out, int64_t dst_stride,
                              cudaStream_t s);

@@ -209,6 +209,10 @@ __global__ void __launch_bounds__(kMsdThreads) msd_partial_kernel(const MsdArgs 
     const bool has_sc = a.scale != nullptr;
     const float sc = has_sc ? a.scale[row] : 1.f;
     const float of = (has_sc && a.offset) ? a.offset[row] : 0.f;
+    if (unit == 0 && tid == 0) {   // what the launches after this one count from
+        if (a.arrived) *a.arrived = 0u;
+        if (a.result) *a.result = spd_result{0ull, 0, 0};
+    }
 
     // 16 samples per thread and step: Eq. 1 on the even and on the odd eight
     // (one per f32x2 lane), Eq. 2 into the lane's running partial
@@ -289,7 +293,12 @@ __device__ __forceinline__ void dmerge(MsdPart &a, const MsdPart &b) {
 __device__ MsdPart block_merge(const MsdPart *parts, int64_t lo, int64_t hi) {
     __shared__ MsdPart s_p[kMsdThreads];
     MsdPart acc{0.0, 0.0, 0.0, 0.0, 0.0};
-    for (int64_t k = lo + threadIdx.x; k < hi; k += kMsdThreads) dmerge(acc, parts[k]);
+    for (int64_t k = lo + threadIdx.x; k < hi; k += kMsdThreads) {
+        const double *d = reinterpret_cast<const double *>(parts + k);   // from L2: maybe written
+        dmerge(acc, MsdPart{__ldcg(d), __ldcg(d + 1), __ldcg(d + 2), __ldcg(d + 3),   // in this
+                            __ldcg(d + 4)});                                         // launch
+    }
+    __syncthreads();   // the last call's result is read
     s_p[threadIdx.x] = acc;
     __syncthreads();
     for (int s = kMsdThreads / 2; s > 0; s >>= 1) {
@@ -325,12 +334,6 @@ __global__ void __launch_bounds__(kMsdThreads) msd_merge_l1_kernel(const MsdPart
     if (threadIdx.x == 0) scratch[blockIdx.x] = r;
 }
 
-__global__ void __launch_bounds__(kMsdThreads) msd_merge_final_kernel(const MsdPart *scratch,
-                                                                      int n, spd_msd_stats *out) {
-    const MsdPart r = block_merge(scratch, 0, n);
-    if (threadIdx.x == 0) write_msd(out, r);
-}
-
 __global__ void __launch_bounds__(kMsdThreads) msd_merge_rows_kernel(const MsdPart *parts,
                                                                      int64_t n_dm, int64_t upr,
                                                                      spd_msd_stats *out) {
@@ -353,19 +356,29 @@ __device__ __forceinline__ int eval_width(const RangeProg &prog, int k) {
     return 0;
 }
 
+__device__ void write_nmax(spd_msd_stats *o, const MsdPart &p, int nmax) {
+    o->nmax = nmax;
+    o->sd_nmax = p.n > 0.0 ? sqrt(p.S / p.n) : 0.0;
+}
+
 // Step (c) constants: per scope entry e and eval index k, 1/sigma_w in FP32
 // (sigma_w in FP64 from Eq. 4 or Eq. 5), and the mean split as hi + lo FP32.
-__global__ void __launch_bounds__(256) consts_kernel(const ConstArgs a,
-                                                     const __grid_constant__ RangeProg prog) {
-    const int e = blockIdx.x;
+// The whole CTA takes part.
+__device__ __forceinline__ void entry_consts(const ConstArgs &a, const RangeProg &prog, int e) {
     const spd_msd_stats m = a.msd[e];
     bool deg = m.status != SPD_OK || !(m.sd > 0.0) || !isfinite(m.sd) || !isfinite(m.mean);
     // Eq. 5 uses the Nmax at which sigma_Nmax was measured (recorded in the MSD).
     const double nm = (double)m.nmax;
     if (a.sigma_mode != SPD_SIGMA_SQRTN && (m.nmax < 2 || !(m.sd_nmax > 0.0) || !isfinite(m.sd_nmax)))
         deg = true;
+    __shared__ int s_imax[kScrTab];
+    if (threadIdx.x < kScrTab) s_imax[threadIdx.x] = 0;
+    if (a.ctl && e == 0 && threadIdx.x < kScrSlots)
+        a.ctl[threadIdx.x] = ScreenCtl{0u, 0u, {0u, 0u}};
+    __syncthreads();
     for (int k = threadIdx.x; k < prog.n_eval; k += blockDim.x) {
-        const double w = (double)eval_width(prog, k);
+        const int wi = eval_width(prog, k);
+        const double w = (double)wi;
         double sw = sqrt(w) * m.sd;
         if (a.sigma_mode == SPD_SIGMA_LINEAR)
             sw += (w - 1.0) * m.sd_nmax / (nm - 1.0);
@@ -373,11 +386,49 @@ __global__ void __launch_bounds__(256) consts_kernel(const ConstArgs a,
             sw += (w - 1.0) * (m.sd_nmax - sqrt(nm) * m.sd) / (nm - 1.0);
         const bool bad = !(sw > 0.0) || !isfinite(sw);
         // a NaN 1/sigma makes every SNR of that width NaN, which no max keeps
-        a.inv_tab[(int64_t)e * prog.n_eval + k] =
-            (a.skip_w1 && k == 0) ? __int_as_float(0x7fc00000) : bad ? 0.f : (float)(1.0 / sw);
+        const bool none = a.skip_w1 && k == 0;
+        const float inv = none ? __int_as_float(0x7fc00000) : bad ? 0.f : (float)(1.0 / sw);
+        a.inv_tab[(int64_t)e * prog.n_eval + k] = inv;
         if (bad) deg = true;
+        if (a.scr_tab && !none && !bad) {   // positive floats order as integers
+            const int c = screen_class(wi);
+            atomicMax(&s_imax[c], __float_as_int(inv));
+            if (c < 2) {
+                const int m2 = __float_as_int((float)wi * inv * inv);
+                if (c == 0) atomicMax(&s_imax[kScrClasses], m2);
+                atomicMax(&s_imax[kScrClasses + 1], m2);
+            }
+        }
     }
-    deg = __syncthreads_or(deg);
+    deg = __syncthreads_or(deg);   // also: inv_tab and s_imax are complete
+    if (a.scr_tab) {
+        // margins for the rounding of the computed SNRs (a few ulp)
+        if (threadIdx.x < kScrTab)
+            a.scr_tab[(int64_t)e * kScrTab + threadIdx.x] =
+                __int_as_float(s_imax[threadIdx.x]) *
+                (threadIdx.x < kScrClasses ? 1.00002f : 1.00004f);
+        // the factors of each group's bounds, as the search kernel forms them:
+        // the second a running max from the narrowest group up
+        __shared__ float s_m2[kMaxCodeGroups];
+        float2 gt = make_float2(0.f, 0.f);
+        if (threadIdx.x < prog.n_groups) {
+            const Group g = prog.groups[threadIdx.x];
+            const int d = (g.flags & kGroupCoarse) ? prog.G : 1;
+            for (int c = 0; c < g.count; ++c) {
+                const float inv = a.inv_tab[(int64_t)e * prog.n_eval + g.widx0 + c];
+                gt.x = fmaxf(gt.x, inv);
+                gt.y = fmaxf(gt.y, (float)(g.off + (c + 1) * d) * inv * inv);
+            }
+            gt.x *= 1.00002f;
+            s_m2[threadIdx.x] = gt.y * 1.00004f;
+        }
+        __syncthreads();
+        if (threadIdx.x < prog.n_groups) {
+            float run = 0.f;
+            for (int g = 0; g <= (int)threadIdx.x; ++g) run = fmaxf(run, s_m2[g]);
+            a.grp_tab[(int64_t)e * prog.n_groups + threadIdx.x] = make_float2(gt.x, run);
+        }
+    }
     if (threadIdx.x == 0) {
         const float hi = (float)m.mean;
         const float lo = (float)(m.mean - (double)hi);
@@ -385,6 +436,49 @@ __global__ void __launch_bounds__(256) consts_kernel(const ConstArgs a,
         a.flags[e] = deg ? 1 : 0;
         if (deg && a.result) atomicExch(&a.result->status, (int)SPD_ERR_DEGENERATE_SIGMA);
     }
+}
+
+__global__ void __launch_bounds__(256) consts_kernel(const ConstArgs a,
+                                                     const __grid_constant__ RangeProg prog) {
+    entry_consts(a, prog, blockIdx.x);
+}
+
+// The merge of n_parts partials in one launch: CTA b folds parts [b per,
+// (b + 1) per) into scratch[b]; the CTA that arrives last folds the scratch
+// (the same fixed tree whichever it is, so the result is deterministic),
+// writes the MSD (nmax 0) or its sigma_Nmax, and forms the constants of the
+// one scope entry when asked for (consts.msd not null).  `arrived` is 0 at
+// launch and again after it.
+//
+// Bound by the latency of its FP64 divisions: 25 us for 32768 parts (4096 x
+// 524288), what the three launches it replaced took without the gaps between
+// them; the searches of 64 x 65536 samples, bound by the host, gain the three
+// launches (a fold, a memset and the constants) it and the partials save.
+__global__ void __launch_bounds__(kMsdThreads)
+    msd_merge_kernel(const MsdPart *parts, int64_t n_parts, int64_t per, MsdPart *scratch,
+                     unsigned *arrived, int nmax, spd_msd_stats *out, const ConstArgs consts,
+                     const __grid_constant__ RangeProg prog) {
+    const int64_t lo = blockIdx.x * per;
+    MsdPart r = block_merge(parts, lo, min(n_parts, lo + per));
+    if (gridDim.x > 1) {
+        __shared__ bool s_last;
+        if (threadIdx.x == 0) {
+            scratch[blockIdx.x] = r;
+            __threadfence();
+            s_last = atomicInc(arrived, gridDim.x - 1) == gridDim.x - 1;
+            __threadfence();
+        }
+        __syncthreads();
+        if (!s_last) return;
+        r = block_merge(scratch, 0, gridDim.x);
+    }
+    if (threadIdx.x == 0) {
+        if (nmax) write_nmax(out, r, nmax);
+        else write_msd(out, r);
+    }
+    if (!consts.msd) return;
+    __syncthreads();
+    entry_consts(consts, prog, 0);
 }
 
 // ----------------------------------------------------- sigma_Nmax (Eq. 5)
@@ -660,18 +754,6 @@ __global__ void __launch_bounds__(kNmaxThreads, 5) nmax_partial_kernel(const Nma
     }
 }
 
-__device__ void write_nmax(spd_msd_stats *o, const MsdPart &p, int nmax) {
-    o->nmax = nmax;
-    o->sd_nmax = p.n > 0.0 ? sqrt(p.S / p.n) : 0.0;
-}
-
-__global__ void __launch_bounds__(kMsdThreads) nmax_merge_final_kernel(const MsdPart *scratch,
-                                                                       int n, int nmax,
-                                                                       spd_msd_stats *out) {
-    const MsdPart r = block_merge(scratch, 0, n);
-    if (threadIdx.x == 0) write_nmax(out, r, nmax);
-}
-
 __global__ void __launch_bounds__(kMsdThreads) nmax_merge_rows_kernel(const MsdPart *parts,
                                                                       int64_t n_dm, int64_t tpr,
                                                                       int nmax, spd_msd_stats *out) {
@@ -756,23 +838,35 @@ cudaError_t launch_msd_partial(const MsdArgs &a, int dtype, cudaStream_t s) {
     return cudaGetLastError();
 }
 
+namespace {
+
+// Global scope: one launch (scratch's last place holds the arrival counter).
+cudaError_t launch_merge(const MsdPart *parts, int64_t n_parts, MsdPart *scratch, int n_scratch,
+                         int nmax, spd_msd_stats *out, const ConstArgs *consts,
+                         const RangeProg *prog, cudaStream_t s) {
+    static const RangeProg none = {};
+    int64_t n1 = (n_parts + kMsdThreads - 1) / kMsdThreads;
+    if (n1 > n_scratch - 1) n1 = n_scratch - 1;
+    if (n1 < 1) n1 = 1;
+    const int64_t per = (n_parts + n1 - 1) / n1;
+    msd_merge_kernel<<<(unsigned)n1, kMsdThreads, 0, s>>>(
+        parts, n_parts, per, scratch, merge_counter(scratch, n_scratch), nmax, out,
+        consts ? *consts : ConstArgs{}, prog ? *prog : none);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
 cudaError_t launch_msd_merge(const MsdPart *parts, int64_t n_dm, int64_t upr, int64_t n_samp,
                              int per_row, MsdPart *scratch, int n_scratch, spd_msd_stats *out,
-                             cudaStream_t s) {
+                             const ConstArgs *consts, const RangeProg *prog, cudaStream_t s) {
     (void)n_samp;
     if (per_row) {
         const unsigned g = (unsigned)((n_dm + kMsdThreads - 1) / kMsdThreads);
         msd_merge_rows_kernel<<<g, kMsdThreads, 0, s>>>(parts, n_dm, upr, out);
         return cudaGetLastError();
     }
-    const int64_t n_parts = n_dm * upr;
-    int64_t n1 = (n_parts + kMsdThreads - 1) / kMsdThreads;
-    if (n1 > n_scratch) n1 = n_scratch;
-    if (n1 < 1) n1 = 1;
-    const int64_t per = (n_parts + n1 - 1) / n1;
-    msd_merge_l1_kernel<<<(unsigned)n1, kMsdThreads, 0, s>>>(parts, n_parts, per, scratch);
-    msd_merge_final_kernel<<<1, kMsdThreads, 0, s>>>(scratch, (int)n1, out);
-    return cudaGetLastError();
+    return launch_merge(parts, n_dm * upr, scratch, n_scratch, 0, out, consts, prog, s);
 }
 
 int nmax_blocks(int nmax) { return (kNmaxTile + nmax + 15) / 16 + 1; }
@@ -821,7 +915,8 @@ cudaError_t launch_merge_shards(const MsdPart *parts, int n, int what, int nmax,
 }
 
 cudaError_t launch_nmax(const NmaxArgs &a, int dtype, MsdPart *scratch, int n_scratch,
-                        spd_msd_stats *out, cudaStream_t s) {
+                        spd_msd_stats *out, const ConstArgs *consts, const RangeProg *prog,
+                        cudaStream_t s) {
     const int64_t tiles = a.n_dm * a.tiles_per_row;
     {
         cudaError_t e = launch_nmax_partial(a, dtype, s);
@@ -832,13 +927,7 @@ cudaError_t launch_nmax(const NmaxArgs &a, int dtype, MsdPart *scratch, int n_sc
         nmax_merge_rows_kernel<<<g, kMsdThreads, 0, s>>>(a.parts, a.n_dm, a.tiles_per_row, a.nmax, out);
         return cudaGetLastError();
     }
-    int64_t n1 = (tiles + kMsdThreads - 1) / kMsdThreads;
-    if (n1 > n_scratch) n1 = n_scratch;
-    if (n1 < 1) n1 = 1;
-    const int64_t per = (tiles + n1 - 1) / n1;
-    msd_merge_l1_kernel<<<(unsigned)n1, kMsdThreads, 0, s>>>(a.parts, tiles, per, scratch);
-    nmax_merge_final_kernel<<<1, kMsdThreads, 0, s>>>(scratch, (int)n1, a.nmax, out);
-    return cudaGetLastError();
+    return launch_merge(a.parts, tiles, scratch, n_scratch, a.nmax, out, consts, prog, s);
 }
 
 cudaError_t launch_stream_msd(const MsdPart *parts, int64_t n_dm, int64_t upr, int per_row,

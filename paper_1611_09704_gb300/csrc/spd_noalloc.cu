@@ -108,11 +108,13 @@ extern "C" spd_status spd_msd_noalloc(const spd_plane *plane, int32_t scope,
         a.vec_ok = (reinterpret_cast<uintptr_t>(plane->data) % need == 0) &&
                    ((size_t)plane->row_stride * spd::elem_bytes(plane->dtype)) % need == 0;
         a.parts = parts;
+        a.arrived = spd::merge_counter(slots, kMergeSlots);
+        a.result = nullptr;
         e = spd::launch_msd_partial(a, plane->dtype, st);
         if (e != cudaSuccess) { spd::note_cuda_error((int)e); return SPD_ERR_CUDA; }
     }
     e = spd::launch_msd_merge(parts, plane->n_dm, upr, plane->n_samp, scope == SPD_MSD_PER_ROW,
-                              slots, kMergeSlots, out_dev, st);
+                              slots, kMergeSlots, out_dev, nullptr, nullptr, st);
     if (e != cudaSuccess) { spd::note_cuda_error((int)e); return SPD_ERR_CUDA; }
     return SPD_OK;
 }

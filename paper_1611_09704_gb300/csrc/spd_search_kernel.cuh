@@ -49,51 +49,11 @@
 // Widths past the row end see y = -inf (sums -inf or NaN), which no max keeps
 // and which no bound prunes wrongly (NaN bounds never prune).
 #pragma once
-#include "spd_device.cuh"
+#include "spd_live.cuh"
 
 namespace spd {
 
 namespace {
-
-__device__ __forceinline__ int sadr(int p) { return (p & 15) + kSPad * (p >> 4); }
-
-// Centred values y = (x - mu.hi) - mu.lo of window positions p .. p+N-1
-// (x = fmaf(scale, q, offset) for scaled storage), -inf at and past `have`.
-// Elements below nraw come from the raw staging buffer, the rest of the row
-// from global memory.
-template <int DT, int N>
-__device__ __forceinline__ void load_centred(float *v, const typename Elem<DT>::T *raw,
-                                             const typename Elem<DT>::T *gsrc, int p, int nraw,
-                                             int have, bool has_sc, float sc, float of, float2 mu) {
-    const float2 mh = make_float2(-mu.x, -mu.x), ml = make_float2(-mu.y, -mu.y);
-    if (p + N <= nraw) {
-#pragma unroll
-        for (int u = 0; u < N / 4; ++u) {
-            float a, b, c, d;
-            load4v<DT>(raw + p + 4 * u, a, b, c, d);
-            float2 x0 = make_float2(a, b), x1 = make_float2(c, d);
-            if (has_sc) {
-                const float2 s2 = make_float2(sc, sc), o2 = make_float2(of, of);
-                x0 = fma2(s2, x0, o2);
-                x1 = fma2(s2, x1, o2);
-            }
-            x0 = add2(add2(x0, mh), ml);
-            x1 = add2(add2(x1, mh), ml);
-            v[4 * u] = x0.x; v[4 * u + 1] = x0.y; v[4 * u + 2] = x1.x; v[4 * u + 3] = x1.y;
-        }
-    } else {
-#pragma unroll
-        for (int e = 0; e < N; ++e) {
-            const int q = p + e;
-            float x = 0.f;
-            if (q < nraw) x = Elem<DT>::cvt(raw[q]);
-            else if (q < have) x = Elem<DT>::cvt(gsrc[q]);
-            if (has_sc) x = fmaf(sc, x, of);
-            x = __fsub_rn(__fsub_rn(x, mu.x), mu.y);
-            v[e] = q < have ? x : -INFINITY;
-        }
-    }
-}
 
 // --------------------------------------------------------- group evaluation
 
@@ -390,14 +350,13 @@ struct TilePos {
 };
 
 template <int DT, int G, bool MG, int NT, bool PL>
-__global__ void __launch_bounds__(NT, 512 / NT) search_kernel(const __grid_constant__ Launch L) {
+__device__ __forceinline__ void search_tiles(const Launch &L, unsigned char *smem) {
     constexpr int kThreads = NT;
     // units of 16 starts per tile: NT less the halo blocks when the whole
     // window then fits one block per thread (one staging round), else NT
     const int U = L.units;
     const int64_t kTile = (int64_t)kX * U;   // starts of one tile
     using T = typename Elem<DT>::T;
-    extern __shared__ __align__(16) unsigned char smem[];
     const int RM = L.R;          // multiple of 4
     const int KM = L.kmax;
     const SearchSmem sm = search_smem(RM, L.raw_bytes, L.max_eval, KM, G);
@@ -444,11 +403,15 @@ __global__ void __launch_bounds__(NT, 512 / NT) search_kernel(const __grid_const
     // search)
     __shared__ long long s_ntiles;
     __shared__ int s_chunk;
+    // with a list (PL: never) `tile` is an index into it, in chunks of one
+    const uint32_t *list = PL ? nullptr : L.tile_list;
     if (tid == 0) {
-        s_ntiles = PL ? (int64_t)(blockIdx.x + 1) * L.n_tiles / gridDim.x : L.n_tiles;
+        s_ntiles = PL ? (int64_t)(blockIdx.x + 1) * L.n_tiles / gridDim.x
+                      : list ? (int64_t)*L.tile_count : L.n_tiles;
         s_chunk = L.chunk;
     }
     __syncthreads();
+    if (list && tile >= s_ntiles) return;   // more CTAs than listed tiles
     // chunks are aligned and a power of two long: a tile is its chunk's last
     // when the next one starts a chunk
     auto chunk_ends = [&]() {
@@ -471,6 +434,17 @@ __global__ void __launch_bounds__(NT, 512 / NT) search_kernel(const __grid_const
     }
     auto pos_of = [&](int64_t t) {
         TilePos p;
+        if (list) {   // tile indexes of a list fit 32 bits (the host checks)
+            const uint32_t tl = list[t];
+            int r = 0;
+            while (r + 1 < L.n_ranges && (int64_t)tl >= L.rng[r + 1].tile0) ++r;
+            const uint32_t lt = tl - (uint32_t)L.rng[r].tile0;
+            const uint32_t q = lt / (uint32_t)L.rng[r].tiles_per_row;
+            p.ri = r;
+            p.row = q;
+            p.col = lt - q * (uint32_t)L.rng[r].tiles_per_row;
+            return p;
+        }
         int r = 0;
         while (r + 1 < L.n_ranges && t >= L.rng[r + 1].tile0) ++r;
         const int64_t lt = t - L.rng[r].tile0;
@@ -1066,6 +1040,20 @@ __global__ void __launch_bounds__(NT, 512 / NT) search_kernel(const __grid_const
     flush();
 }
 
+// The tiles, then (after a screen) the live units of the tiles not searched
+// whole.
+template <int DT, int G, bool MG, int NT, bool PL>
+__global__ void __launch_bounds__(NT, 512 / NT) search_kernel(const __grid_constant__ Launch L) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    search_tiles<DT, G, MG, NT, PL>(L, smem);
+    if constexpr (!PL && NT == kSearchThreads) {
+        if (L.unit_list) {
+            __syncthreads();
+            live_units<DT, G, MG>(L, reinterpret_cast<float *>(smem));
+        }
+    }
+}
+
 template <int DT, int G, int NT, bool PL>
 cudaError_t launch_sgn(const Launch &L, bool mg, size_t smem, int ctas_per_sm, cudaStream_t s) {
     int dev = 0, sms = 0, per_sm = 0;
@@ -1086,7 +1074,7 @@ cudaError_t launch_sgn(const Launch &L, bool mg, size_t smem, int ctas_per_sm, c
     const int64_t gmax = (int64_t)sms * per_sm;
     int64_t ch = 16;
     while (ch > 1 && L.n_tiles < 8 * gmax * ch) ch >>= 1;
-    if (PL) ch = 1;
+    if (PL || L.tile_list) ch = 1;
     Launch Lc = L;
     Lc.chunk = (int32_t)ch;
     const int64_t n_chunks = (L.n_tiles + ch - 1) / ch;
