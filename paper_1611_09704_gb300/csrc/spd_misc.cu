@@ -126,24 +126,33 @@ __global__ void boxcar_sums_kernel(const spd_plane p, int w, float *out, int64_t
     *o = s;
 }
 
-// Per-DM clustering of the candidates (snr >= thr) in time: one warp scans
-// one row, 32 samples per step, kClusterSteps steps of loads in flight.  In
-// sample order a candidate joins the open cluster when it lies at most `gap`
-// samples after the previous candidate, else the open cluster is written and
-// a new one starts.  A step is taken a segment at a time, not a candidate at a
-// time: each lane finds its previous candidate (in the step's ballot mask, or
-// the open cluster's last), the lanes that start a cluster form a second mask,
-// and each segment between starts is absorbed with a popcount, its highest
-// set bit, and one warp max (redux) over order-preserving keys of its SNRs.
-// Every lane holds the same cluster state, so lane 0 alone writes records.
-constexpr int kClusterWarps = 8;   // rows per CTA
-constexpr int kClusterSteps = 8;   // 32-sample steps loaded at once per warp
+// Per-DM clustering of the candidates of an SNR plane.  A row is cut into
+// segments, a warp each; a cluster belongs to the segment of its first
+// candidate.  Its warp follows it past the segment's end; a warp whose
+// segment begins inside a cluster (a candidate at most `gap` before its first
+// one, found by looking back) passes over the rest of that one.  So the
+// records are those of one walk along the whole row.
+//
+// A step is 32 consecutive samples, one per lane; 16 steps are loaded at once,
+// and with no candidate among them are done with one vote.  In a step the
+// candidates are a ballot mask, the lanes that start a cluster (more than
+// `gap` past the last candidate before them: the previous set bit, else the
+// open cluster's last) form a second mask, and each segment between starts is
+// absorbed with a popcount, its highest set bit, and one warp max (redux)
+// over order-preserving keys of its SNRs.  Every lane holds the same cluster
+// state, so lane 0 alone writes records, and reads the peak's width then: the
+// width plane is not streamed.
+//
+// Bound by the SNR plane's one read.  1024 x 262144 samples: a warp per row
+// left 7 warps per SM and streamed the widths too, 815 us; now 169 us, 6.3
+// TB/s.
+constexpr int kClusterWarps = 8;    // segments per CTA
+constexpr int kClusterSteps = 16;   // 32-sample steps loaded at once per warp
 
 struct ClusterState {
-    int64_t first, last, peak_t, members;
+    int first, last, peak_t, members;
     float peak;
     unsigned peak_key;
-    int peak_w;
 };
 
 // Monotone map of a non-NaN float to an unsigned key (larger float, larger
@@ -156,20 +165,20 @@ __device__ __forceinline__ unsigned order_key(float f) {
 }
 
 __device__ __forceinline__ void emit_cluster(const ClusterState &c, int64_t row,
-                                             spd_cluster *out, int64_t capacity,
-                                             spd_result *result, int lane) {
+                                             const uint16_t *wp, spd_cluster *out,
+                                             int64_t capacity, spd_result *result, int lane) {
     if (lane != 0) return;
     const unsigned long long idx =
         atomicAdd(reinterpret_cast<unsigned long long *>(&result->count), 1ull);
     if (idx < (unsigned long long)capacity) {
         spd_cluster r;
         r.dm = (int32_t)row;
-        r.first = (int32_t)c.first;
-        r.last = (int32_t)c.last;
-        r.peak_sample = (int32_t)c.peak_t;
+        r.first = c.first;
+        r.last = c.last;
+        r.peak_sample = c.peak_t;
         r.peak_snr = c.peak;
-        r.peak_width = c.peak_w;
-        r.members = (int32_t)c.members;
+        r.peak_width = wp[c.peak_t];
+        r.members = c.members;
         r.reserved0 = 0;
         out[idx] = r;
     }
@@ -178,8 +187,8 @@ __device__ __forceinline__ void emit_cluster(const ClusterState &c, int64_t row,
 // The members M (a lane mask of this step, starting at sample t0) join the
 // open cluster: count, last sample, and the peak (strict: an earlier equal
 // peak stays; within M the lowest lane of the maximum).
-__device__ __forceinline__ void absorb(ClusterState &c, unsigned M, int64_t t0, unsigned key,
-                                       float v, int w, int lane) {
+__device__ __forceinline__ void absorb(ClusterState &c, unsigned M, int t0, unsigned key, float v,
+                                       int lane) {
     c.members += __popc(M);
     c.last = t0 + (31 - __clz(M));
     const unsigned mine = ((M >> lane) & 1u) ? key : 0u;
@@ -188,62 +197,83 @@ __device__ __forceinline__ void absorb(ClusterState &c, unsigned M, int64_t t0, 
         const int pl = __ffs(__ballot_sync(0xffffffffu, mine == kmax)) - 1;
         c.peak_key = kmax;
         c.peak = __shfl_sync(0xffffffffu, v, pl);
-        c.peak_w = __shfl_sync(0xffffffffu, w, pl);
         c.peak_t = t0 + pl;
     }
 }
 
 __global__ void __launch_bounds__(32 * kClusterWarps) cluster_kernel(
-    const float *snr, const uint16_t *width, int64_t n_dm, int64_t n_samp, int64_t stride,
-    float thr, int64_t gap, spd_cluster *out, int64_t capacity, spd_result *result) {
+    const float *snr, const uint16_t *width, int n_dm, int n, int64_t stride, float thr, int gap,
+    int seg_len, int segs_per_row, spd_cluster *out, int64_t capacity, spd_result *result) {
     const int lane = threadIdx.x & 31;
-    const int64_t row = (int64_t)blockIdx.x * kClusterWarps + (threadIdx.x >> 5);
+    const int64_t sg = (int64_t)blockIdx.x * kClusterWarps + (threadIdx.x >> 5);
+    const int64_t row = sg / segs_per_row;
     if (row >= n_dm) return;   // the whole warp
+    const int a = (int)(sg - row * segs_per_row) * seg_len;
+    const int b = n - a < seg_len ? n : a + seg_len;
     const float *sp = snr + row * stride;
     const uint16_t *wp = width + row * stride;
-    bool open = false;
-    ClusterState c{0, 0, 0, 0, 0.f, 0u, 0};
-    for (int64_t base = 0; base < n_samp; base += 32 * kClusterSteps) {
+    bool open = false, foreign = false, looked = a == 0;
+    ClusterState c{0, 0, 0, 0, 0.f, 0u};
+    // the segment, then on past its end while an own cluster is open
+    for (int64_t base = a; base < n; base += 32 * kClusterSteps) {
+        if (base >= b && (!open || foreign || base - c.last > gap)) break;
         float v[kClusterSteps];
-        int w[kClusterSteps];
+        bool any = false;
 #pragma unroll
         for (int k = 0; k < kClusterSteps; ++k) {
             const int64_t t = base + 32 * k + lane;
-            v[k] = t < n_samp ? __ldcs(sp + t) : -INFINITY;
-            w[k] = t < n_samp ? (int)__ldcs(wp + t) : 0;
+            v[k] = t < n ? __ldcs(sp + t) : -INFINITY;
         }
 #pragma unroll
+        for (int k = 0; k < kClusterSteps; ++k) any |= v[k] >= thr;   // NaN: not a candidate
+        if (!__any_sync(0xffffffffu, any)) continue;
+#pragma unroll
         for (int k = 0; k < kClusterSteps; ++k) {
-            const bool cand = v[k] >= thr;   // NaN: not a candidate
+            const bool cand = v[k] >= thr && base + 32 * k + lane < n;
             const unsigned m = __ballot_sync(0xffffffffu, cand);
             if (!m) continue;
-            const int64_t t0 = base + 32 * k;
+            const int t0 = (int)(base + 32 * k);
+            if (!looked) {   // the segment's first candidate: in a cluster from before it?
+                looked = true;
+                const int t1 = t0 + __ffs(m) - 1;
+                for (int q = a; q > 0 && t1 - (q - 1) <= gap && !foreign; q -= 32) {
+                    const int p = q - 32 + lane;
+                    const bool hit = p >= 0 && t1 - p <= gap && sp[p] >= thr;
+                    foreign = __any_sync(0xffffffffu, hit);
+                }
+                if (foreign) {
+                    open = true;
+                    c.last = t1 - 1;   // any sample at most gap before it
+                }
+            }
             // does this lane's candidate start a cluster?
             const unsigned below = m & ((1u << lane) - 1u);
             const bool has_prev = below != 0u || open;
-            const int64_t prev = below ? t0 + (31 - __clz(below)) : c.last;
+            const int prev = below ? t0 + (31 - __clz(below)) : c.last;
             const bool start = cand && (!has_prev || (t0 + lane) - prev > gap);
             unsigned S = __ballot_sync(0xffffffffu, start);
             const unsigned key = cand ? order_key(v[k]) : 0u;
             // members before the first start continue the open cluster
             const int fs = S ? __ffs(S) - 1 : 32;
             const unsigned cont = fs == 32 ? m : (m & ((1u << fs) - 1u));
-            if (cont) absorb(c, cont, t0, key, v[k], w[k], lane);
+            if (cont) absorb(c, cont, t0, key, v[k], lane);
             while (S) {
                 const int s0 = __ffs(S) - 1;
                 S &= S - 1u;
                 const int e = S ? __ffs(S) - 1 : 32;
                 const unsigned seg = m & (0xffffffffu << s0) & (e == 32 ? 0xffffffffu : ((1u << e) - 1u));
-                if (open) emit_cluster(c, row, out, capacity, result, lane);
-                open = true;
+                if (open && !foreign) emit_cluster(c, row, wp, out, capacity, result, lane);
+                open = t0 + s0 < b;   // one that starts past the segment is the next one's
+                foreign = false;
+                if (!open) return;
                 c.first = t0 + s0;
                 c.members = 0;
                 c.peak_key = 0u;
-                absorb(c, seg, t0, key, v[k], w[k], lane);
+                absorb(c, seg, t0, key, v[k], lane);
             }
         }
     }
-    if (open) emit_cluster(c, row, out, capacity, result, lane);
+    if (open && !foreign) emit_cluster(c, row, wp, out, capacity, result, lane);
 }
 
 }  // namespace
@@ -382,10 +412,21 @@ cudaError_t launch_cluster(const float *snr, const uint16_t *width, int64_t n_dm
                            int64_t n_samp, int64_t stride, float thr, int64_t gap,
                            spd_cluster *out, int64_t capacity, spd_result *result,
                            cudaStream_t s) {
-    const int64_t blocks = (n_dm + kClusterWarps - 1) / kClusterWarps;
-    if (blocks <= 0 || n_samp <= 0) return cudaSuccess;
+    if (n_dm <= 0 || n_samp <= 0) return cudaSuccess;
+    // segments: about 32768 (200 per SM), of at least 4096 samples (a warp's
+    // fixed work is that of some 512) and at least 4 gaps (looking back reads
+    // one)
+    const int64_t step = 32 * kClusterSteps;
+    if (gap > n_samp) gap = n_samp;
+    int64_t len = (n_dm * n_samp / 32768 + step - 1) / step * step;
+    if (len < 4096) len = 4096;
+    if (len < 4 * gap) len = (4 * gap + step - 1) / step * step;
+    if (len > n_samp) len = n_samp;
+    const int64_t per_row = (n_samp + len - 1) / len;
+    const int64_t blocks = (n_dm * per_row + kClusterWarps - 1) / kClusterWarps;
     cluster_kernel<<<(unsigned)blocks, 32 * kClusterWarps, 0, s>>>(
-        snr, width, n_dm, n_samp, stride, thr, gap, out, capacity, result);
+        snr, width, (int)n_dm, (int)n_samp, stride, thr, (int)gap, (int)len, (int)per_row, out,
+        capacity, result);
     return cudaGetLastError();
 }
 
