@@ -512,7 +512,8 @@ spd_status spd_debug_set_copy_wait(uint64_t limit_ns, uint32_t extra_bytes);
  * trials straight into a streaming search's chunk view
  * (spd_stream_chunk_view) and the push reads them in place:
  *   out[d][t] = sum over channels c of x[c][t + delays[d * n_chan + c]],
- * t < n_out, summed in FP32 in channel order.
+ * t < n_out, summed in FP32 in channel order (two neighbouring channels may
+ * be summed first).
  * fb: the filterbank as a plane of n_chan = fb->n_dm channel rows of
  * fb->n_samp samples (any storage type, with optional per-channel scale and
  * offset as for the search).  delays: device int32 [n_dm][n_chan] in samples,
