@@ -368,7 +368,8 @@ spd_status run_launch(const RangeDesc *rd, int n, int dtype, spd_candidate *out,
                       const ScreenLists *lists = nullptr) {
     static thread_local Launch L;
     memset(&L, 0, sizeof(L));
-    const int nt = !snr_out && (threads == 128 || threads == 256) ? threads : kSearchThreads;
+    const int nt = snr_out ? kPlaneThreads
+                   : threads == 128 || threads == 256 ? threads : kSearchThreads;
     // candidate search: U units of 16 starts per tile, the threads less the
     // widest range's halo blocks when that leaves one block per thread
     int halo = 0;
@@ -412,7 +413,7 @@ spd_status run_launch(const RangeDesc *rd, int n, int dtype, spd_candidate *out,
     L.extra_tx = g_extra_tx;
     // plane output (every sample's best SNR and width) evaluates every group
     // and needs no bound tables
-    int kmax = 0;
+    int kmax = snr_out ? -1 : 0;
     for (int i = 0; i < n && !snr_out; ++i) {
         const int k = prog_kmax(rd[i].prog);
         kmax = k > kmax ? k : kmax;

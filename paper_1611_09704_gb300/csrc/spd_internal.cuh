@@ -206,24 +206,26 @@ __host__ __device__ inline GroupGeom group_geom(int off, int count, int d) {
 struct SearchSmem {
     size_t raw, y, p, g, bs, mx, mn, pq, ex, eq, rh, rl, inv, gr, ew, total;
 };
+// Plane output (kmax < 0) has no bounds: no array from mx to rl.
 __host__ __device__ inline SearchSmem search_smem(int RM, int raw_bytes, int max_eval, int kmax,
                                                   int G) {
     SearchSmem m;
     const size_t blk = (size_t)kSPad * RM * sizeof(float);
     const size_t arr = (size_t)RM * sizeof(float);
+    const size_t bnd = kmax < 0 ? 0 : arr;
     m.raw = 16;
     m.y = m.raw + (size_t)raw_bytes;
     m.p = m.y + blk;
     m.g = m.p + blk;
     m.bs = m.g + (G > 1 ? blk : 0);
     m.mx = m.bs + arr;                       // level 0; levels 1..kmax follow
-    m.mn = m.mx + (size_t)(1 + kmax) * arr;
-    m.pq = m.mn + arr;
-    m.ex = m.pq + arr + 16;
-    m.eq = m.ex + arr;
-    m.rh = m.eq + arr;
-    m.rl = m.rh + arr;
-    m.inv = m.rl + arr;
+    m.mn = m.mx + (size_t)(1 + kmax) * arr;   // kmax -1: nothing
+    m.pq = m.mn + bnd;
+    m.ex = m.pq + bnd + 16;
+    m.eq = m.ex + bnd;
+    m.rh = m.eq + bnd;
+    m.rl = m.rh + bnd;
+    m.inv = m.rl + bnd;
     m.gr = m.inv + (((size_t)max_eval * sizeof(float) + 15) & ~(size_t)15);
     m.ew = m.gr + (size_t)kMaxCodeGroups * 32;
     m.total = (m.ew + (size_t)max_eval * sizeof(uint16_t) + 15) & ~(size_t)15;
@@ -330,6 +332,7 @@ cudaError_t launch_nmax(const NmaxArgs &a, int dtype, MsdPart *scratch, int n_sc
 cudaError_t launch_search(const Launch &L, int dtype, int G, bool multi_block, size_t smem,
                           int ctas_per_sm, int threads, cudaStream_t s);
 constexpr int kSearchThreads = 256;   // threads of a search CTA by default
+constexpr int kPlaneThreads = 256;    // threads of a plane-output CTA
 // The screen of a launch's ranges (geometry as for launch_search).
 cudaError_t launch_screen(const Launch &L, const ScreenLists &S, int dtype, cudaStream_t s);
 // x[2j] + x[2j+1] of a plane (dequantised) into an FP32 plane, j < n_out.

@@ -671,7 +671,9 @@ __device__ __forceinline__ void search_tiles(const Launch &L, unsigned char *sme
                 }
                 hi = fmaxf(hi, Cp[15]);
                 lo = fminf(lo, Cp[15]);
-                if (16 * c + 16 <= have) {
+                if (PL) {
+                    // no bounds: neither the extrema nor the energy
+                } else if (16 * c + 16 <= have) {
                     float2 e2 = make_float2(0.f, 0.f);
 #pragma unroll
                     for (int q = 0; q < 8; ++q) {
@@ -703,9 +705,12 @@ __device__ __forceinline__ void search_tiles(const Launch &L, unsigned char *sme
                     }
                 }
                 s_bs[c] = sum;
-                s_rh[c] = hi;
-                s_rl[c] = lo;
+                if (!PL) {
+                    s_rh[c] = hi;
+                    s_rl[c] = lo;
+                }
             }
+            if (PL) continue;
             // inclusive warp scans of the block sums and energies; exclusive
             // values by shuffle (the block holding the window's end has sum
             // -inf, yet the prefix at its start is finite)
@@ -804,11 +809,11 @@ __device__ __forceinline__ void search_tiles(const Launch &L, unsigned char *sme
 
         // ---- search of the unit's 16 starts (widest group first)
         const float thr = rd.threshold;
-        const float minC = s_mn[tid];
+        const float minC = PL ? 0.f : s_mn[tid];
         // the FP32 prefix values are off by at most ~30 roundings of the
         // tile's largest partial sum: the prefix bound adds twice that
         const float cslack = fmaf(8e-6f, __int_as_float(s_mag), 1e-30f) - minC;
-        const float pq0 = s_pq[tid];
+        const float pq0 = PL ? 0.f : s_pq[tid];
         const float *yb = s_y + kSPad * tid;
         float cb[kX];
         float ob[MG ? kX : 1];
@@ -1087,7 +1092,7 @@ cudaError_t launch_sgn(const Launch &L, bool mg, size_t smem, int ctas_per_sm, c
 template <int DT, int G>
 cudaError_t launch_sg(const Launch &L, bool mg, size_t smem, int ctas_per_sm, int threads,
                       cudaStream_t s) {
-    if (L.snr_out) return launch_sgn<DT, G, 256, true>(L, mg, smem, ctas_per_sm, s);
+    if (L.snr_out) return launch_sgn<DT, G, kPlaneThreads, true>(L, mg, smem, ctas_per_sm, s);
     return threads == 128 ? launch_sgn<DT, G, 128, false>(L, mg, smem, ctas_per_sm, s)
                           : launch_sgn<DT, G, 256, false>(L, mg, smem, ctas_per_sm, s);
 }
