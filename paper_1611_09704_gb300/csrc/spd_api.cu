@@ -1155,12 +1155,14 @@ spd_status check_info(const spd_stream_info *info, const StreamLayout &S, int32_
     return SPD_OK;
 }
 
-// Search the combined buffer [halo | chunk] (n = halo + chunk samples per row)
-// with the running MSD in `stats`; emit starts below n_emit.
+// The running MSD with the chunk's unit partials (upr per row; none at a flush)
+// added, then the search of the combined buffer [halo | chunk] (n = halo +
+// chunk samples per row) with it; emits starts below n_emit.
 spd_status stream_search(const spd_stream_info *info, const RangeProg &prog,
                          const spd_search_params *params, const void *comb, int64_t cstride,
                          int64_t n, int64_t n_emit, const float *scale, const float *offset,
-                         const spd_msd_stats *stats, spd_candidate *out, int64_t cap,
+                         MsdPart *parts, int64_t upr, MsdPart *scratch, MsdPart *run,
+                         spd_msd_stats *stats, spd_candidate *out, int64_t cap,
                          spd_result *result, void *det_ws, char *scr, cudaStream_t st) {
     spd_plane cp;
     memset(&cp, 0, sizeof(cp));
@@ -1171,15 +1173,33 @@ spd_status stream_search(const spd_stream_info *info, const RangeProg &prog,
     cp.row_stride = cstride;
     cp.row_scale = scale;
     cp.row_offset = offset;
-    RangeDesc rd;
     const int64_t tiles = screen_tiles(info->n_dm, cstride);
     const ScreenLists lists = lists_at(scr, tiles);
-    SPD_TRY(range_consts(&cp, prog, stats, params->msd_scope, params->sigma_mode, result, det_ws,
-                         st, rd, 0, scr ? scr + screen_lists(tiles).total : nullptr, lists.ctl));
+    const ConstArgs c = const_args(&cp, prog, stats, params->msd_scope, params->sigma_mode, result,
+                                   det_ws, 0, scr ? scr + screen_lists(tiles).total : nullptr,
+                                   lists.ctl);
+    const bool rows = params->msd_scope == SPD_MSD_PER_ROW;
+    SPD_CK(launch_stream_msd(parts, info->n_dm, upr, rows, run, scratch, kMergeScratch, stats,
+                             rows ? nullptr : &c, &prog, st));
+    if (rows) SPD_CK(launch_consts(c, prog, st));
+    RangeDesc rd = range_desc(&cp, prog, params->msd_scope, c);
     rd.threshold = params->threshold;
     rd.n_emit = n_emit;
     rd.sample_base = info->seen - info->halo;
     return run_launch(&rd, 1, info->dtype, out, cap, result, nullptr, nullptr, 0, 0, st, 0, &lists);
+}
+
+// Memory of the current device: kernels may read it as they do a workspace.
+// Anything else (page-locked or pageable host memory, managed memory, another
+// device's) goes through the runtime's copies.
+bool on_this_device(const void *p) {
+    int dev = 0;
+    cudaPointerAttributes a;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice && a.device == dev;
 }
 
 }  // namespace
@@ -1250,8 +1270,10 @@ spd_status spd_stream_push(spd_stream_info *info, void *state_dev, const spd_pla
     char *halo = state + S.halo_off;
     char *comb = ws + P.comb_off;
     const int64_t H = info->halo;
-    SPD_CK(cudaMemsetAsync(result_dev, 0, sizeof(spd_result), st));
-    if (L == 0) return SPD_OK;
+    if (L == 0) {
+        SPD_CK(cudaMemsetAsync(result_dev, 0, sizeof(spd_result), st));
+        return SPD_OK;
+    }
     if (info->seen == 0) {
         // the flush has no chunk: keep the beam's scale / offset in the state
         const size_t rb = (size_t)info->n_dm * sizeof(float);
@@ -1265,53 +1287,57 @@ spd_status spd_stream_push(spd_stream_info *info, void *state_dev, const spd_pla
         info->has_offset = chunk->row_offset != nullptr;
     }
     // [halo | chunk] into the combined buffer
+    const int64_t cb = P.cstride * (int64_t)eb;
     if (H > 0)
-        SPD_CK(cudaMemcpy2DAsync(comb, P.cstride * eb, halo, S.halo_cap * eb, H * eb, info->n_dm,
-                                 cudaMemcpyDeviceToDevice, st));
+        SPD_CK(launch_copy_rows(comb, cb, halo, S.halo_cap * eb, H * eb, info->n_dm, (int)eb, st));
     const char *src = static_cast<const char *>(chunk->data);
+    spd_plane in_place = *chunk;   // the chunk where the MSD reads it
     if (src == comb + H * eb && chunk->row_stride == P.cstride) {
         // written in place through spd_stream_chunk_view
     } else if (src < ws + workspace_bytes && src + (size_t)chunk->n_dm * chunk->row_stride * eb > ws) {
         return SPD_ERR_INVALID_ARG;  // inside the workspace but not at the view
+    } else if (on_this_device(src)) {
+        // the MSD reads the chunk itself: its rows may lie on vector
+        // boundaries where those of the combined buffer do not
+        SPD_CK(launch_copy_rows(comb + H * eb, cb, src, chunk->row_stride * (int64_t)eb, L * eb,
+                                info->n_dm, (int)eb, st));
     } else {
-        // device or page-locked host memory (unified addressing decides)
+        // page-locked or pageable host memory (unified addressing decides)
         SPD_CK(cudaMemcpy2DAsync(comb + H * eb, P.cstride * eb, src, chunk->row_stride * eb,
                                  L * eb, info->n_dm, cudaMemcpyDefault, st));
+        in_place.data = comb + H * eb;
+        in_place.row_stride = P.cstride;
     }
-    // running MSD: the chunk's unit partials (read from its place in the
-    // combined buffer) added to the state
-    spd_plane in_place = *chunk;
-    in_place.data = comb + H * eb;
-    in_place.row_stride = P.cstride;
+    // running MSD: the chunk's unit partials, added to the state below
     const MsdLayout ML = msd_layout(&in_place);
+    MsdPart *parts = reinterpret_cast<MsdPart *>(ws + P.msd_off + ML.parts_off);
+    MsdPart *scratch = reinterpret_cast<MsdPart *>(ws + P.msd_off + ML.scratch_off);
     MsdArgs ma;
     ma.data = in_place.data;
     ma.n_dm = chunk->n_dm;
     ma.n_samp = L;
-    ma.stride = P.cstride;
+    ma.stride = in_place.row_stride;
     ma.scale = chunk->row_scale;
     ma.offset = chunk->row_offset;
     ma.units_per_row = ML.upr;
     ma.vec_ok = plane_vec_ok(&in_place);
-    MsdPart *parts = reinterpret_cast<MsdPart *>(ws + P.msd_off);
     ma.parts = parts;
-    ma.arrived = nullptr;
-    ma.result = nullptr;
+    ma.arrived = merge_counter(scratch, kMergeScratch);
+    ma.result = result_dev;
     SPD_CK(launch_msd_partial(ma, chunk->dtype, st));
     spd_msd_stats *stats =
         msd_out_dev ? msd_out_dev : reinterpret_cast<spd_msd_stats *>(ws + P.stats_off);
-    SPD_CK(launch_stream_msd(parts, info->n_dm, ML.upr, params->msd_scope == SPD_MSD_PER_ROW,
-                             run, stats, st));
     // search every start with a full window; hold the last wmax - 1 back
     const int64_t n = H + L;
     const int64_t hold = n < (int64_t)(prog.wmax - 1) ? n : (int64_t)(prog.wmax - 1);
     const int64_t n_emit = n - hold;
     SPD_TRY(stream_search(info, prog, params, comb, P.cstride, n, n_emit, chunk->row_scale,
-                          chunk->row_offset, stats, out, capacity, result_dev, ws + P.det_off,
+                          chunk->row_offset, parts, ML.upr, scratch, run, stats, out, capacity,
+                          result_dev, ws + P.det_off,
                           screen_at(workspace, workspace_bytes, P.total, P.scr_bytes), st));
     if (hold > 0)
-        SPD_CK(cudaMemcpy2DAsync(halo, S.halo_cap * eb, comb + n_emit * eb, P.cstride * eb,
-                                 hold * eb, info->n_dm, cudaMemcpyDeviceToDevice, st));
+        SPD_CK(launch_copy_rows(halo, S.halo_cap * eb, comb + n_emit * eb, cb, hold * eb,
+                                info->n_dm, (int)eb, st));
     info->seen += L;
     info->halo = hold;
     info->chunks += 1;
@@ -1354,18 +1380,23 @@ spd_status spd_stream_flush(spd_stream_info *info, void *state_dev,
     const size_t eb = elem_bytes(info->dtype);
     char *ws = static_cast<char *>(workspace);
     char *state = static_cast<char *>(state_dev);
-    SPD_CK(cudaMemcpy2DAsync(ws + P.comb_off, P.cstride * eb, state + S.halo_off,
-                             S.halo_cap * eb, H * eb, info->n_dm, cudaMemcpyDeviceToDevice, st));
+    SPD_CK(launch_copy_rows(ws + P.comb_off, P.cstride * (int64_t)eb, state + S.halo_off,
+                            S.halo_cap * (int64_t)eb, H * eb, info->n_dm, (int)eb, st));
+    spd_plane probe;
+    memset(&probe, 0, sizeof(probe));
+    probe.n_dm = info->n_dm;
+    probe.n_samp = 1;
+    const MsdLayout ML = msd_layout(&probe);
+    MsdPart *parts = reinterpret_cast<MsdPart *>(ws + P.msd_off + ML.parts_off);
+    MsdPart *scratch = reinterpret_cast<MsdPart *>(ws + P.msd_off + ML.scratch_off);
     spd_msd_stats *stats = reinterpret_cast<spd_msd_stats *>(ws + P.stats_off);
-    SPD_CK(launch_stream_msd(reinterpret_cast<MsdPart *>(ws + P.msd_off), info->n_dm, 0,
-                             info->msd_scope == SPD_MSD_PER_ROW,
-                             reinterpret_cast<MsdPart *>(state + S.msd_off), stats, st));
     const float *scale = info->has_scale ? reinterpret_cast<const float *>(state + S.scale_off)
                                          : nullptr;
     const float *offset = info->has_offset
                               ? reinterpret_cast<const float *>(state + S.offset_off)
                               : nullptr;
     SPD_TRY(stream_search(info, prog, params, ws + P.comb_off, P.cstride, H, H, scale, offset,
+                          parts, 0, scratch, reinterpret_cast<MsdPart *>(state + S.msd_off),
                           stats, out, capacity, result_dev, ws + P.det_off,
                           screen_at(workspace, workspace_bytes, P.total, P.scr_bytes), st));
     info->halo = 0;

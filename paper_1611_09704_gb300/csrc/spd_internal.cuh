@@ -312,7 +312,12 @@ cudaError_t launch_msd_merge(const MsdPart *parts, int64_t n_dm, int64_t units_p
 // too.  The partials' launch has set merge_counter(scratch, n_scratch) to 0.
 cudaError_t launch_consts(const ConstArgs &a, const RangeProg &prog, cudaStream_t s);
 cudaError_t launch_stream_msd(const MsdPart *parts, int64_t n_dm, int64_t upr, int per_row,
-                              MsdPart *state, spd_msd_stats *out, cudaStream_t s);
+                              MsdPart *state, MsdPart *scratch, int n_scratch, spd_msd_stats *out,
+                              const ConstArgs *consts, const RangeProg *prog, cudaStream_t s);
+// width bytes (a multiple of esz, 2 or 4) of each of n_rows rows.  Addresses
+// and row strides are multiples of esz; all device memory.
+cudaError_t launch_copy_rows(void *dst, int64_t dst_stride, const void *src, int64_t src_stride,
+                             int64_t width, int64_t n_rows, int esz, cudaStream_t s);
 cudaError_t launch_zero_parts(MsdPart *p, int64_t n, cudaStream_t s);
 int nmax_blocks(int nmax);
 // sigma_Nmax partials per row (CTAs of the partial kernel per row).

@@ -345,6 +345,66 @@ cudaError_t launch_threshold_plane(float *snr, uint16_t *width, int64_t n_dm, in
     return cudaGetLastError();
 }
 
+// Rows of a halo or a chunk from one pitch to another, where the two may lie
+// differently to 16-byte boundaries (a stream's halo is wmax - 1 samples long,
+// so its chunk follows at any element step).  One 16-byte piece of the
+// destination per thread: from one piece of the source or, shifted, from the
+// two it lies in; the pieces at a row's ends, and those whose source pieces
+// stick out of the source, element by element.  2048 x 32768 FP16 at an odd
+// step: a 2-D copy by the runtime took 0.1 ms, this 0.04.
+template <typename T>
+__global__ void __launch_bounds__(256) copy_rows_kernel(char *dst, int64_t dst_stride,
+                                                        const char *src, int64_t src_stride,
+                                                        int64_t width, int64_t pieces,
+                                                        int64_t n_rows) {
+    const int64_t idx = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    const int64_t row = gridDim.x < (1u << 24) ? (uint32_t)idx / (uint32_t)pieces : idx / pieces;
+    if (row >= n_rows) return;
+    char *d0 = dst + row * dst_stride;
+    const char *s0 = src + row * src_stride;
+    const char *end = src + (n_rows - 1) * src_stride + width;
+    // the piece's first byte, from the row's start (negative: before it)
+    const int64_t o = (idx - row * pieces) * 16 - (int64_t)(reinterpret_cast<uintptr_t>(d0) & 15);
+    if (o >= width) return;
+    const char *p = s0 + o;
+    const uint32_t m = (uint32_t)(reinterpret_cast<uintptr_t>(p) & 15);
+    if (o >= 0 && o + 16 <= width && p - m >= src && p - m + (m ? 32 : 16) <= end) {
+        uint4 a = __ldg(reinterpret_cast<const uint4 *>(p - m));
+        if (m) {
+            const uint4 b = __ldg(reinterpret_cast<const uint4 *>(p - m) + 1);
+            uint32_t w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+            const uint32_t k = m >> 2, half = (m & 2) * 8u;
+#pragma unroll
+            for (int i = 0; i < 7; ++i) w[i] = (k & 1) ? w[i + 1] : w[i];
+#pragma unroll
+            for (int i = 0; i < 6; ++i) w[i] = (k & 2) ? w[i + 2] : w[i];
+            a = make_uint4(__funnelshift_r(w[0], w[1], half), __funnelshift_r(w[1], w[2], half),
+                           __funnelshift_r(w[2], w[3], half), __funnelshift_r(w[3], w[4], half));
+        }
+        *reinterpret_cast<uint4 *>(d0 + o) = a;
+        return;
+    }
+    for (int64_t e = o < 0 ? 0 : o; e < o + 16 && e < width; e += (int64_t)sizeof(T))
+        *reinterpret_cast<T *>(d0 + e) = *reinterpret_cast<const T *>(s0 + e);
+}
+
+cudaError_t launch_copy_rows(void *dst, int64_t dst_stride, const void *src, int64_t src_stride,
+                             int64_t width, int64_t n_rows, int esz, cudaStream_t s) {
+    if (width <= 0 || n_rows <= 0) return cudaSuccess;
+    const int64_t pieces = width / 16 + 2;   // a row may begin and end inside one
+    const int64_t blocks = (n_rows * pieces + 255) / 256;
+    if (blocks > INT32_MAX) return cudaErrorInvalidValue;
+    char *d = static_cast<char *>(dst);
+    const char *p = static_cast<const char *>(src);
+    if (esz == 2)
+        copy_rows_kernel<uint16_t><<<(unsigned)blocks, 256, 0, s>>>(d, dst_stride, p, src_stride,
+                                                                    width, pieces, n_rows);
+    else
+        copy_rows_kernel<uint32_t><<<(unsigned)blocks, 256, 0, s>>>(d, dst_stride, p, src_stride,
+                                                                    width, pieces, n_rows);
+    return cudaGetLastError();
+}
+
 // Decimation in time by 2: dst[r][j] = x[r][2j] + x[r][2j+1] in FP32 (x the
 // dequantised source), for j < n_out.  Four outputs per thread.
 template <int DT>

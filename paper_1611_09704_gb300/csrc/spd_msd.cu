@@ -493,7 +493,7 @@ __global__ void __launch_bounds__(256) consts_kernel(const ConstArgs a,
 // (the same fixed tree whichever it is, so the result is deterministic),
 // writes the MSD (nmax 0) or its sigma_Nmax, and forms the constants of the
 // one scope entry when asked for (consts.msd not null).  `arrived` is 0 at
-// launch and again after it.
+// launch and again after it.  With `state` the parts join a running MSD.
 //
 // Bound by the latency of its FP64 divisions: 25 us for 32768 parts (4096 x
 // 524288), what the three launches it replaced took without the gaps between
@@ -501,8 +501,8 @@ __global__ void __launch_bounds__(256) consts_kernel(const ConstArgs a,
 // launches (a fold, a memset and the constants) it and the partials save.
 __global__ void __launch_bounds__(kMsdThreads)
     msd_merge_kernel(const MsdPart *parts, int64_t n_parts, int64_t per, MsdPart *scratch,
-                     unsigned *arrived, int nmax, spd_msd_stats *out, const ConstArgs consts,
-                     const __grid_constant__ RangeProg prog) {
+                     unsigned *arrived, int nmax, MsdPart *state, spd_msd_stats *out,
+                     const ConstArgs consts, const __grid_constant__ RangeProg prog) {
     const int64_t lo = blockIdx.x * per;
     MsdPart r = block_merge(parts, lo, min(n_parts, lo + per));
     if (gridDim.x > 1) {
@@ -518,6 +518,12 @@ __global__ void __launch_bounds__(kMsdThreads)
         r = block_merge(scratch, 0, gridDim.x);
     }
     if (threadIdx.x == 0) {
+        if (state) {   // a stream's running MSD: the state first, then this chunk
+            MsdPart run = *state;
+            dmerge(run, r);
+            *state = run;
+            r = run;
+        }
         if (nmax) write_nmax(out, r, nmax);
         else write_msd(out, r);
     }
@@ -837,21 +843,8 @@ __global__ void merge_shards_kernel(const MsdPart *parts, int n, int what, int n
 // Running MSD of a stream: state[e] holds (n, T, S, min, max) of every sample
 // pushed so far for scope entry e.  The new chunk's unit partials are added
 // with Eq. 2 (state first, then the chunk in unit order) and the result is
-// written back and as spd_msd_stats.  Global scope: one CTA; per row: one
-// thread per row.
-__global__ void __launch_bounds__(kMsdThreads) stream_msd_global_kernel(const MsdPart *parts,
-                                                                       int64_t n_parts,
-                                                                       MsdPart *state,
-                                                                       spd_msd_stats *out) {
-    const MsdPart c = block_merge(parts, 0, n_parts);
-    if (threadIdx.x == 0) {
-        MsdPart s = *state;
-        dmerge(s, c);
-        *state = s;
-        write_msd(out, s);
-    }
-}
-
+// written back and as spd_msd_stats.  Global scope: msd_merge_kernel; per row:
+// one thread per row.
 __global__ void __launch_bounds__(kMsdThreads) stream_msd_rows_kernel(const MsdPart *parts,
                                                                      int64_t n_dm, int64_t upr,
                                                                      MsdPart *state,
@@ -887,7 +880,7 @@ namespace {
 
 // Global scope: one launch (scratch's last place holds the arrival counter).
 cudaError_t launch_merge(const MsdPart *parts, int64_t n_parts, MsdPart *scratch, int n_scratch,
-                         int nmax, spd_msd_stats *out, const ConstArgs *consts,
+                         int nmax, MsdPart *state, spd_msd_stats *out, const ConstArgs *consts,
                          const RangeProg *prog, cudaStream_t s) {
     static const RangeProg none = {};
     int64_t n1 = (n_parts + kMsdThreads - 1) / kMsdThreads;
@@ -895,7 +888,7 @@ cudaError_t launch_merge(const MsdPart *parts, int64_t n_parts, MsdPart *scratch
     if (n1 < 1) n1 = 1;
     const int64_t per = (n_parts + n1 - 1) / n1;
     msd_merge_kernel<<<(unsigned)n1, kMsdThreads, 0, s>>>(
-        parts, n_parts, per, scratch, merge_counter(scratch, n_scratch), nmax, out,
+        parts, n_parts, per, scratch, merge_counter(scratch, n_scratch), nmax, state, out,
         consts ? *consts : ConstArgs{}, prog ? *prog : none);
     return cudaGetLastError();
 }
@@ -911,7 +904,7 @@ cudaError_t launch_msd_merge(const MsdPart *parts, int64_t n_dm, int64_t upr, in
         msd_merge_rows_kernel<<<g, kMsdThreads, 0, s>>>(parts, n_dm, upr, out);
         return cudaGetLastError();
     }
-    return launch_merge(parts, n_dm * upr, scratch, n_scratch, 0, out, consts, prog, s);
+    return launch_merge(parts, n_dm * upr, scratch, n_scratch, 0, nullptr, out, consts, prog, s);
 }
 
 int nmax_blocks(int nmax) { return (kNmaxTile + nmax + 15) / 16 + 1; }
@@ -972,18 +965,18 @@ cudaError_t launch_nmax(const NmaxArgs &a, int dtype, MsdPart *scratch, int n_sc
         nmax_merge_rows_kernel<<<g, kMsdThreads, 0, s>>>(a.parts, a.n_dm, a.tiles_per_row, a.nmax, out);
         return cudaGetLastError();
     }
-    return launch_merge(a.parts, tiles, scratch, n_scratch, a.nmax, out, consts, prog, s);
+    return launch_merge(a.parts, tiles, scratch, n_scratch, a.nmax, nullptr, out, consts, prog, s);
 }
 
 cudaError_t launch_stream_msd(const MsdPart *parts, int64_t n_dm, int64_t upr, int per_row,
-                              MsdPart *state, spd_msd_stats *out, cudaStream_t s) {
+                              MsdPart *state, MsdPart *scratch, int n_scratch, spd_msd_stats *out,
+                              const ConstArgs *consts, const RangeProg *prog, cudaStream_t s) {
     if (per_row) {
         const unsigned g = (unsigned)((n_dm + kMsdThreads - 1) / kMsdThreads);
         if (g) stream_msd_rows_kernel<<<g, kMsdThreads, 0, s>>>(parts, n_dm, upr, state, out);
-    } else {
-        stream_msd_global_kernel<<<1, kMsdThreads, 0, s>>>(parts, n_dm * upr, state, out);
+        return cudaGetLastError();
     }
-    return cudaGetLastError();
+    return launch_merge(parts, n_dm * upr, scratch, n_scratch, 0, state, out, consts, prog, s);
 }
 
 cudaError_t launch_zero_parts(MsdPart *p, int64_t n, cudaStream_t s) {
