@@ -1070,22 +1070,30 @@ spd_status spd_search_decimated(const spd_plane *plane, const spd_level *levels,
     SPD_TRY(dec_plan(plane, levels, n_levels, threshold, ranges, shifts, D, base));
     SPD_TRY(check_ws(workspace, workspace_bytes, D.total));
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    // level l from level l - 1 (the input plane for l = 1)
-    for (int l = 1; l <= D.lmax; ++l) {
+    // levels l + 1 .. l + 4 from level l (the input plane for l = 0); of these
+    // only what is searched, or decimated further, is stored
+    for (int l = 0; l < D.lmax; l += 4) {
         spd_plane src;
-        if (l == 1) {
+        if (l == 0) {
             src = *plane;
         } else {
             memset(&src, 0, sizeof(src));
-            src.data = base + D.plane_off[l - 1];
+            src.data = base + D.plane_off[l];
             src.dtype = SPD_F32;
             src.n_dm = plane->n_dm;
-            src.n_samp = D.n[l - 1];
-            src.row_stride = D.stride[l - 1];
+            src.n_samp = D.n[l];
+            src.row_stride = D.stride[l];
         }
-        if (!plane_empty(&src))
-            SPD_CK(launch_decimate2(src, reinterpret_cast<float *>(base + D.plane_off[l]), D.n[l],
-                                    D.stride[l], st));
+        const int m = D.lmax - l < 4 ? D.lmax - l : 4;
+        float *dst[4] = {nullptr, nullptr, nullptr, nullptr};
+        int64_t stride[4] = {0, 0, 0, 0};
+        for (int k = 0; k < m; ++k) {
+            bool wanted = k == 3 && l + 4 < D.lmax;
+            for (int i = 0; i < n_levels; ++i) wanted = wanted || levels[i].level == l + k + 1;
+            if (wanted) dst[k] = reinterpret_cast<float *>(base + D.plane_off[l + k + 1]);
+            stride[k] = D.stride[l + k + 1];
+        }
+        if (!plane_empty(&src)) SPD_CK(launch_decimate(src, dst, stride, m, st));
     }
     return batched_impl(ranges, n_levels, nullptr, shifts, out, capacity, result_dev, msd_out_dev,
                         base + D.batch_off, workspace_bytes - D.batch_off, stream);

@@ -340,9 +340,11 @@ constexpr int kSearchThreads = 256;   // threads of a search CTA by default
 constexpr int kPlaneThreads = 256;    // threads of a plane-output CTA
 // The screen of a launch's ranges (geometry as for launch_search).
 cudaError_t launch_screen(const Launch &L, const ScreenLists &S, int dtype, cudaStream_t s);
-// x[2j] + x[2j+1] of a plane (dequantised) into an FP32 plane, j < n_out.
-cudaError_t launch_decimate2(const spd_plane &p, float *dst, int64_t n_out, int64_t dst_stride,
-                             cudaStream_t s);
+// Levels 1 .. `levels` (at most 4) of decimation by 2 of a plane (dequantised)
+// into FP32 planes of 16-byte aligned rows: dst[k] (null: not wanted) holds
+// n_samp >> (k + 1) sums of 2^(k+1) samples per row.
+cudaError_t launch_decimate(const spd_plane &p, float *const *dst, const int64_t *stride,
+                            int levels, cudaStream_t s);
 cudaError_t launch_threshold_plane(float *snr, uint16_t *width, int64_t n_dm, int64_t n_samp,
                                    int64_t stride, float thr, cudaStream_t s);
 cudaError_t launch_threshold(const float *snr, const uint16_t *width, int64_t n_dm,

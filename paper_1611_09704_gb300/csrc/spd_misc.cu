@@ -405,61 +405,96 @@ cudaError_t launch_copy_rows(void *dst, int64_t dst_stride, const void *src, int
     return cudaGetLastError();
 }
 
-// Decimation in time by 2: dst[r][j] = x[r][2j] + x[r][2j+1] in FP32 (x the
-// dequantised source), for j < n_out.  Four outputs per thread.
+// Decimation in time: up to four levels of a plane in one pass, level k + 1
+// from level k: dst_k[r][j] = dst_{k-1}[r][2j] + dst_{k-1}[r][2j+1] in FP32
+// (dst_-1: the dequantised source).  A thread sums 16 consecutive source
+// samples to 8, 4, 2 and 1 outputs.  Level by level, 1024 x 262144 FP32 down
+// to 1/16 read 2.0 GB and took 492 us; this reads the source once.
+struct DecimateArgs {
+    const void *src;
+    int64_t src_stride, n_src;
+    const float *scale, *offset;
+    float *dst[4];              // null: not wanted
+    int64_t stride[4], n[4];    // n[k] = n_src >> (k + 1)
+    int vec_ok;                 // 16-byte aligned rows
+};
+
 template <int DT>
-__global__ void __launch_bounds__(256) decimate2_kernel(const typename Elem<DT>::T *src,
-                                                        int64_t src_stride, const float *scale,
-                                                        const float *offset, int64_t n_out,
-                                                        float *dst, int64_t dst_stride) {
+__global__ void __launch_bounds__(256) decimate_kernel(const __grid_constant__ DecimateArgs a) {
+    using T = typename Elem<DT>::T;
     const int64_t row = blockIdx.y;
-    const int64_t j0 = ((int64_t)blockIdx.x * 256 + threadIdx.x) * 4;
-    if (j0 >= n_out) return;
-    const typename Elem<DT>::T *sp = src + row * src_stride + 2 * j0;
-    const float sc = scale ? scale[row] : 1.f;
-    const float of = (scale && offset) ? offset[row] : 0.f;
-    float o[4];
+    const int64_t t = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    const int64_t i0 = 16 * t;
+    if (i0 >= a.n_src) return;
+    const T *sp = static_cast<const T *>(a.src) + row * a.src_stride + i0;
+    float v[16];
+    if (a.vec_ok && i0 + 16 <= a.n_src) {
+        constexpr int kVec = DT == SPD_F32 ? 4 : 2;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        if (j0 + q < n_out) {
-            float a = Elem<DT>::cvt(sp[2 * q]), b = Elem<DT>::cvt(sp[2 * q + 1]);
-            if (scale) { a = fmaf(sc, a, of); b = fmaf(sc, b, of); }
-            o[q] = __fadd_rn(a, b);
+        for (int q = 0; q < kVec; ++q) {
+            const uint4 u = __ldg(reinterpret_cast<const uint4 *>(sp) + q);
+            const T *e = reinterpret_cast<const T *>(&u);
+#pragma unroll
+            for (int k = 0; k < 16 / kVec; ++k) v[16 / kVec * q + k] = Elem<DT>::cvt(e[k]);
         }
-    }
-    float *dp = dst + row * dst_stride + j0;
-    if (j0 + 4 <= n_out && (reinterpret_cast<uintptr_t>(dp) & 15) == 0) {
-        *reinterpret_cast<float4 *>(dp) = make_float4(o[0], o[1], o[2], o[3]);
     } else {
-        for (int q = 0; q < 4 && j0 + q < n_out; ++q) dp[q] = o[q];
+#pragma unroll
+        for (int q = 0; q < 16; ++q) v[q] = i0 + q < a.n_src ? Elem<DT>::cvt(sp[q]) : 0.f;
+    }
+    if (a.scale) {
+        const float sc = a.scale[row], of = a.offset ? a.offset[row] : 0.f;
+#pragma unroll
+        for (int q = 0; q < 16; ++q) v[q] = fmaf(sc, v[q], of);
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int m = 8 >> k;              // outputs of this level
+#pragma unroll
+        for (int q = 0; q < m; ++q) v[q] = __fadd_rn(v[2 * q], v[2 * q + 1]);
+        if (!a.dst[k]) continue;
+        const int64_t j0 = t * m;
+        float *d = a.dst[k] + row * a.stride[k] + j0;
+        if (j0 + m <= a.n[k]) {
+            if (m >= 4) {
+#pragma unroll
+                for (int q = 0; q < m; q += 4)
+                    *reinterpret_cast<float4 *>(d + q) = make_float4(v[q], v[q + 1], v[q + 2], v[q + 3]);
+            } else if (m == 2) {
+                *reinterpret_cast<float2 *>(d) = make_float2(v[0], v[1]);
+            } else {
+                *d = v[0];
+            }
+        } else {
+#pragma unroll
+            for (int q = 0; q < m; ++q)
+                if (j0 + q < a.n[k]) d[q] = v[q];
+        }
     }
 }
 
-cudaError_t launch_decimate2(const spd_plane &p, float *dst, int64_t n_out, int64_t dst_stride,
-                             cudaStream_t s) {
-    if (p.n_dm <= 0 || n_out <= 0) return cudaSuccess;
+cudaError_t launch_decimate(const spd_plane &p, float *const *dst, const int64_t *stride, int levels,
+                            cudaStream_t s) {
+    if (p.n_dm <= 0 || p.n_samp < 2) return cudaSuccess;
     for (int64_t r0 = 0; r0 < p.n_dm; r0 += 65535) {   // grid.y limit
         const int64_t y = p.n_dm - r0 < 65535 ? p.n_dm - r0 : 65535;
-        const dim3 grid((unsigned)((n_out + 1023) / 1024), (unsigned)y);
-        const float *sc = p.row_scale ? p.row_scale + r0 : nullptr;
-        const float *of = p.row_offset ? p.row_offset + r0 : nullptr;
-        float *d = dst + r0 * dst_stride;
+        const size_t eb = elem_bytes(p.dtype);
+        DecimateArgs a;
+        a.src = static_cast<const char *>(p.data) + r0 * p.row_stride * (int64_t)eb;
+        a.src_stride = p.row_stride;
+        a.n_src = p.n_samp;
+        a.scale = p.row_scale ? p.row_scale + r0 : nullptr;
+        a.offset = p.row_offset ? p.row_offset + r0 : nullptr;
+        for (int k = 0; k < 4; ++k) {
+            a.dst[k] = k < levels && dst[k] ? dst[k] + r0 * stride[k] : nullptr;
+            a.stride[k] = k < levels ? stride[k] : 0;
+            a.n[k] = p.n_samp >> (k + 1);
+        }
+        a.vec_ok = reinterpret_cast<uintptr_t>(a.src) % 16 == 0 && (p.row_stride * (int64_t)eb) % 16 == 0;
+        const dim3 grid((unsigned)((p.n_samp + 4095) / 4096), (unsigned)y);
         switch (p.dtype) {
-            case SPD_F32:
-                decimate2_kernel<SPD_F32><<<grid, 256, 0, s>>>(
-                    static_cast<const float *>(p.data) + r0 * p.row_stride, p.row_stride, sc, of,
-                    n_out, d, dst_stride);
-                break;
-            case SPD_F16:
-                decimate2_kernel<SPD_F16><<<grid, 256, 0, s>>>(
-                    static_cast<const __half *>(p.data) + r0 * p.row_stride, p.row_stride, sc, of,
-                    n_out, d, dst_stride);
-                break;
-            default:
-                decimate2_kernel<SPD_BF16><<<grid, 256, 0, s>>>(
-                    static_cast<const __nv_bfloat16 *>(p.data) + r0 * p.row_stride, p.row_stride,
-                    sc, of, n_out, d, dst_stride);
-                break;
+            case SPD_F32: decimate_kernel<SPD_F32><<<grid, 256, 0, s>>>(a); break;
+            case SPD_F16: decimate_kernel<SPD_F16><<<grid, 256, 0, s>>>(a); break;
+            default: decimate_kernel<SPD_BF16><<<grid, 256, 0, s>>>(a); break;
         }
     }
     return cudaGetLastError();
