@@ -339,24 +339,87 @@ __device__ __forceinline__ void dmerge(MsdPart &a, const MsdPart &b) {
     a.n = a.n + b.n;
 }
 
-// Block-wide Eq. 2 over parts[lo, hi): thread t folds lo+t, lo+t+256, ... in
-// order, then a halving tree in shared memory.  Result valid in thread 0.
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+    for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// Eq. 2 over parts[lo, hi) by the CTA: thread t folds lo+t, lo+t+256, ... in
+// order; the threads' sets are merged at once, as n = sum n_t, T = sum T_t and
+// S = sum S_t + (T_t - n_t T / n)^2 / n_t -- Eq. 2 applied to all of them,
+// whose terms are non-negative, so nothing cancels.  A fixed order of sums:
+// deterministic.  Result valid in thread 0.
+//
+// An FP64 instruction of a warp takes its SM's FP64 unit 16 cycles, and a
+// division some dozen of them, so eight warps' pairwise folds over eight
+// levels took most of the merge.  Here a thread has about 13: counts are
+// summed as integers, extrema (which are FP32 values) in FP32, T / n is formed
+// once, and 1 / n_t is exact in FP32 where n_t is a power of two, as that of a
+// whole unit is.
 __device__ MsdPart block_merge(const MsdPart *parts, int64_t lo, int64_t hi) {
-    __shared__ MsdPart s_p[kMsdThreads];
+    constexpr int kWarps = kMsdThreads / 32;
+    __shared__ double s_t[kWarps], s_s[kWarps], s_mean;
+    __shared__ long long s_n[kWarps];
+    __shared__ float2 s_r[kWarps];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     MsdPart acc{0.0, 0.0, 0.0, 0.0, 0.0};
     for (int64_t k = lo + threadIdx.x; k < hi; k += kMsdThreads) {
         const double *d = reinterpret_cast<const double *>(parts + k);   // from L2: maybe written
-        dmerge(acc, MsdPart{__ldcg(d), __ldcg(d + 1), __ldcg(d + 2), __ldcg(d + 3),   // in this
-                            __ldcg(d + 4)});                                         // launch
+        const MsdPart p{__ldcg(d), __ldcg(d + 1), __ldcg(d + 2), __ldcg(d + 3),   // in this
+                        __ldcg(d + 4)};                                          // launch
+        if (k == lo + threadIdx.x) acc = p;
+        else dmerge(acc, p);
     }
-    __syncthreads();   // the last call's result is read
-    s_p[threadIdx.x] = acc;
+    long long n = (long long)acc.n;
+    float mn = n ? (float)acc.lo : INFINITY, mx = n ? (float)acc.hi : -INFINITY;
+#pragma unroll
+    for (int o = 16; o; o >>= 1) {
+        n += __shfl_xor_sync(0xffffffffu, n, o);
+        mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    }
+    const double t = warp_sum(acc.T);
+    __syncthreads();   // the last call's results are read
+    if (lane == 0) {
+        s_n[warp] = n;
+        s_t[warp] = t;
+        s_r[warp] = make_float2(mn, mx);
+    }
     __syncthreads();
-    for (int s = kMsdThreads / 2; s > 0; s >>= 1) {
-        if ((int)threadIdx.x < s) dmerge(s_p[threadIdx.x], s_p[threadIdx.x + s]);
-        __syncthreads();
+    MsdPart r{0.0, 0.0, 0.0, 0.0, 0.0};
+    if (threadIdx.x == 0) {
+        n = 0;
+        mn = INFINITY;
+        mx = -INFINITY;
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) {
+            n += s_n[w];
+            r.T += s_t[w];
+            mn = fminf(mn, s_r[w].x);
+            mx = fmaxf(mx, s_r[w].y);
+        }
+        r.n = (double)n;
+        r.lo = n ? (double)mn : 0.0;
+        r.hi = n ? (double)mx : 0.0;
+        s_mean = n ? r.T / r.n : 0.0;
     }
-    return s_p[0];
+    __syncthreads();
+    double q = 0.0;
+    if (acc.n > 0.0) {
+        const double d = fma(-acc.n, s_mean, acc.T);
+        const long long m = (long long)acc.n;
+        if ((m & (m - 1)) == 0) q = fma(d * d, (double)(1.f / (float)m), acc.S);
+        else q = acc.S + d * d / acc.n;
+    }
+    q = warp_sum(q);
+    if (lane == 0) s_s[warp] = q;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) r.S += s_s[w];
+    }
+    return r;
 }
 
 __device__ void write_msd(spd_msd_stats *o, const MsdPart &p) {
@@ -423,6 +486,8 @@ __device__ __forceinline__ void entry_consts(const ConstArgs &a, const RangeProg
     if (a.sigma_mode != SPD_SIGMA_SQRTN && (m.nmax < 2 || !(m.sd_nmax > 0.0) || !isfinite(m.sd_nmax)))
         deg = true;
     __shared__ int s_imax[kScrTab];
+    constexpr int kHeld = 1024;      // 1/sigma_w kept for the groups' factors below
+    __shared__ float s_inv[kHeld];
     if (threadIdx.x < kScrTab) s_imax[threadIdx.x] = 0;
     if (a.ctl && e == 0 && threadIdx.x < kScrSlots)
         a.ctl[threadIdx.x] = ScreenCtl{0u, 0u, {0u, 0u}};
@@ -440,6 +505,7 @@ __device__ __forceinline__ void entry_consts(const ConstArgs &a, const RangeProg
         const bool none = a.skip_w1 && k == 0;
         const float inv = none ? __int_as_float(0x7fc00000) : bad ? 0.f : (float)(1.0 / sw);
         a.inv_tab[(int64_t)e * prog.n_eval + k] = inv;
+        if (k < kHeld) s_inv[k] = inv;
         if (bad) deg = true;
         if (a.scr_tab && !none && !bad) {   // positive floats order as integers
             const int c = screen_class(wi);
@@ -466,7 +532,8 @@ __device__ __forceinline__ void entry_consts(const ConstArgs &a, const RangeProg
             const Group g = prog.groups[threadIdx.x];
             const int d = (g.flags & kGroupCoarse) ? prog.G : 1;
             for (int c = 0; c < g.count; ++c) {
-                const float inv = a.inv_tab[(int64_t)e * prog.n_eval + g.widx0 + c];
+                const int k = g.widx0 + c;
+                const float inv = k < kHeld ? s_inv[k] : a.inv_tab[(int64_t)e * prog.n_eval + k];
                 gt.x = fmaxf(gt.x, inv);
                 gt.y = fmaxf(gt.y, (float)(g.off + (c + 1) * d) * inv * inv);
             }
@@ -589,14 +656,17 @@ __host__ __device__ __forceinline__ int nmax_ywords(int nb) {
 }
 size_t nmax_smem_bytes(int nb) { return ((size_t)nmax_ywords(nb) + nb) * sizeof(float); }
 
-__device__ __forceinline__ float block_sum(const float *s_y, int b) {
+__device__ __forceinline__ float sum16(const float *p) {
     float sum = 0.f;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-        const float4 f = *reinterpret_cast<const float4 *>(s_y + npad(16 * b) + 4 * q);
+        const float4 f = *reinterpret_cast<const float4 *>(p + 4 * q);
         sum += (f.x + f.y) + (f.z + f.w);
     }
     return sum;
+}
+__device__ __forceinline__ float block_sum(const float *s_y, int b) {
+    return sum16(s_y + npad(16 * b));
 }
 
 // Sec. 2.2, Eq. 5 needs sigma_Nmax, the measured sd of the boxcar series
@@ -638,6 +708,14 @@ __global__ void __launch_bounds__(kNmaxThreads, 5) nmax_partial_kernel(const Nma
     const int nmax = a.nmax;
     const int b0 = tid * (kNmaxPer / 16);          // the thread's first block (tile-local)
     const int qe = 16 * b0 + nmax;                 // end of its first window
+    // addresses that do not change from tile to tile: the thread's own run of
+    // 64 positions, where it stages (4 positions of each 512), and from its
+    // run to the 16 samples that enter the window of each quarter
+    const float *own = s_y + npad(kNmaxPer * tid);
+    float *put = s_y + npad(4 * tid);
+    int enter[kNmaxPer / 16];
+#pragma unroll
+    for (int c = 0; c < kNmaxPer / 16; ++c) enter[c] = npad(16 * c + nmax);
     Acc run_acc;    // the thread's runs: one Eq. 2 merge per tile
     for (int64_t tl = tl0; tl < tl1; ++tl) {
         const int64_t t0 = tl * (int64_t)kNmaxTile;
@@ -651,21 +729,20 @@ __global__ void __launch_bounds__(kNmaxThreads, 5) nmax_partial_kernel(const Nma
             const int cq = min(c0 + kQ * kNmaxThreads, nq);   // this round's end
             if (a.vec_ok && t0 + 4 * (int64_t)cq <= a.n_samp) {
                 typename Quad<DT>::V r[kQ];
+                const T *gp = rp + t0 + 4 * (c0 + tid);
+                float *sp = put + npad(4 * c0);   // c0: a multiple of 16
+                const int left = cq - c0 - tid;
+#pragma unroll
+                for (int u = 0; u < kQ; ++u)
+                    if (u * kNmaxThreads < left) r[u] = Quad<DT>::ld(gp + 4 * u * kNmaxThreads);
 #pragma unroll
                 for (int u = 0; u < kQ; ++u) {
-                    const int q4 = c0 + u * kNmaxThreads + tid;
-                    if (q4 < cq) r[u] = Quad<DT>::ld(rp + t0 + 4 * q4);
-                }
-#pragma unroll
-                for (int u = 0; u < kQ; ++u) {
-                    const int q4 = c0 + u * kNmaxThreads + tid;
-                    if (q4 < cq) {
+                    if (u * kNmaxThreads < left) {
                         float2 v0, v1;
                         Quad<DT>::cvt(r[u], v0, v1);
                         v0 = __ffma2_rn(sc2, v0, c2);
                         v1 = __ffma2_rn(sc2, v1, c2);
-                        const int p = 4 * q4;
-                        *reinterpret_cast<float4 *>(s_y + npad(p)) =
+                        *reinterpret_cast<float4 *>(sp + u * npad(4 * kNmaxThreads)) =
                             make_float4(v0.x, v0.y, v1.x, v1.y);
                     }
                 }
@@ -688,7 +765,7 @@ __global__ void __launch_bounds__(kNmaxThreads, 5) nmax_partial_kernel(const Nma
         {
             float bs4[4];
 #pragma unroll
-            for (int c = 0; c < 4; ++c) bs4[c] = block_sum(s_y, b0 + c);
+            for (int c = 0; c < 4; ++c) bs4[c] = sum16(own + 16 * c);
             *reinterpret_cast<float4 *>(s_bs + b0) = make_float4(bs4[0], bs4[1], bs4[2], bs4[3]);
             for (int b = kNmaxTile / 16 + tid; b < a.nb; b += kNmaxThreads)
                 s_bs[b] = block_sum(s_y, b);
@@ -721,51 +798,52 @@ __global__ void __launch_bounds__(kNmaxThreads, 5) nmax_partial_kernel(const Nma
         float2 Td = f2(0.f), Sd = f2(0.f);
         int nrun = 0;
         // starts t0 + 16 b0 + k are full windows while k < nvalid
-        const int64_t nvalid = a.n_samp - nmax - (t0 + 16 * b0) + 1;
-#pragma unroll 1
-        for (int c = 0; c < kNmaxPer / 16; ++c) {
-            // the unit's 16 samples and the 16 that enter the window as it slides
-            const int bl = b0 + c;
-            float lo[16], hi[16];
+        const int64_t nv64 = a.n_samp - nmax - (t0 + 16 * b0) + 1;
+        const int nvalid = nv64 < 0 ? 0 : nv64 < kNmaxPer ? (int)nv64 : kNmaxPer;
+        // the unit's 16 samples and the 16 that enter the window as it slides;
+        // d slides by hi - lo per start (the differences as f32x2 pairs)
+        auto slide = [&](int c, float2 (&bw)[8]) {   // bw[k] = d at unit starts 2k, 2k + 1
+            const float *lp = own + 16 * c;
+            const float *hp = own + enter[c];
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                const float4 f = *reinterpret_cast<const float4 *>(s_y + npad(16 * bl) + 4 * q);
-                lo[4 * q] = f.x; lo[4 * q + 1] = f.y; lo[4 * q + 2] = f.z; lo[4 * q + 3] = f.w;
-            }
-            if ((nmax & 15) == 0) {
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const float4 f =
-                        *reinterpret_cast<const float4 *>(s_y + npad(16 * bl + nmax) + 4 * q);
-                    hi[4 * q] = f.x; hi[4 * q + 1] = f.y; hi[4 * q + 2] = f.z; hi[4 * q + 3] = f.w;
+                const float4 lo = *reinterpret_cast<const float4 *>(lp + 4 * q);
+                float4 hi;
+                if ((nmax & 15) == 0) {
+                    hi = *reinterpret_cast<const float4 *>(hp + 4 * q);
+                } else {
+                    const int p = kNmaxPer * tid + 16 * c + 4 * q + nmax;
+                    hi = make_float4(s_y[npad(p)], s_y[npad(p + 1)], s_y[npad(p + 2)],
+                                     s_y[npad(p + 3)]);
                 }
-            } else {
-#pragma unroll
-                for (int k = 0; k < 16; ++k) {
-                    const int q = 16 * bl + k + nmax;
-                    hi[k] = s_y[npad(q)];
-                }
+                const float2 m1 = f2(-1.f);
+                const float2 da = __ffma2_rn(make_float2(lo.x, lo.y), m1, make_float2(hi.x, hi.y));
+                const float2 db = __ffma2_rn(make_float2(lo.z, lo.w), m1, make_float2(hi.z, hi.w));
+                bw[2 * q].x = Bd;
+                bw[2 * q].y = bw[2 * q].x + da.x;
+                bw[2 * q + 1].x = bw[2 * q].y + da.y;
+                bw[2 * q + 1].y = bw[2 * q + 1].x + db.x;
+                Bd = bw[2 * q + 1].y + db.y;
             }
-            // d slides by hi - lo per start (the differences as f32x2 pairs)
-            float2 bw[8];   // bw[k] = (d at unit start + 2k, d at unit start + 2k + 1)
+        };
+        if (nvalid == kNmaxPer) {
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                const float2 dl = __ffma2_rn(make_float2(lo[2 * k], lo[2 * k + 1]), f2(-1.f),
-                                             make_float2(hi[2 * k], hi[2 * k + 1]));
-                bw[k].x = Bd;
-                Bd += dl.x;
-                bw[k].y = Bd;
-                Bd += dl.y;
-            }
-            const int64_t nv = nvalid - 16 * c;
-            if (nv >= 16) {
+            for (int c = 0; c < kNmaxPer / 16; ++c) {
+                float2 bw[8];
+                slide(c, bw);
 #pragma unroll
                 for (int k = 0; k < 8; ++k) {
                     Td = __fadd2_rn(Td, bw[k]);
                     Sd = __ffma2_rn(bw[k], bw[k], Sd);
                 }
-                nrun += 16;
-            } else if (nv > 0) {   // near the row end: the starts with full windows
+            }
+            nrun = kNmaxPer;
+        } else {   // near the row end: the starts with full windows
+#pragma unroll 1
+            for (int c = 0; 16 * c < nvalid; ++c) {
+                const int nv = nvalid - 16 * c;
+                float2 bw[8];
+                slide(c, bw);
 #pragma unroll
                 for (int k = 0; k < 8; ++k) {
                     const float2 dm = make_float2(2 * k < nv ? bw[k].x : 0.f,
@@ -773,8 +851,8 @@ __global__ void __launch_bounds__(kNmaxThreads, 5) nmax_partial_kernel(const Nma
                     Td = __fadd2_rn(Td, dm);
                     Sd = __ffma2_rn(dm, dm, Sd);
                 }
-                nrun += (int)nv;
             }
+            nrun = nvalid;
         }
         if (nrun) {   // the run's (n, T, S), T with the product n B0 kept exactly
             const float n = (float)nrun;
