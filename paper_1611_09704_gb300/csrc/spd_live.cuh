@@ -25,9 +25,10 @@ __device__ __forceinline__ float half_min(float v, uint32_t hm) {
 // takes its widths one after the other.  Many units in flight hide it: 20 us
 // for the live units of 4096 x 524288 samples of noise.
 //
-// s_dyn: the CTA's dynamic shared memory, whose first use is over.
+// s_dyn: the CTA's dynamic shared memory, whose first use is over.  in_tiles:
+// the units of the listed tiles, when these are searched here too (else 0).
 template <int DT, int G, bool MG>
-__device__ __forceinline__ void live_units(const Launch &L, float *s_dyn) {
+__device__ __forceinline__ void live_units(const Launch &L, float *s_dyn, uint32_t in_tiles) {
     using T = typename Elem<DT>::T;
     const int blocks = L.live_blocks, halves = L.live_halves;
     const uint64_t *units = L.unit_list;
@@ -41,13 +42,20 @@ __device__ __forceinline__ void live_units(const Launch &L, float *s_dyn) {
     float *s_bs = s_p + (G > 1 ? 2 : 1) * blocks * kSPad;
     float *s_mx = s_bs + blocks;
     float *s_pq = s_mx + blocks;                        // [blocks + 1]
-    const uint32_t n = min(*L.unit_count, L.unit_cap);
+    const uint32_t n = in_tiles + min(*L.unit_count, L.unit_cap);
     const uint32_t per = gridDim.x * (uint32_t)halves;
     // warp-uniform trip count: the first half-warp of the warp decides
     for (uint32_t i0 = blockIdx.x * (uint32_t)halves + (uint32_t)((tid >> 5) * 2); i0 < n; i0 += per) {
         const uint32_t i = i0 + (uint32_t)((lane >> 4) & 1);
         uint64_t id = ~0ull;
-        if (has_room && i < n) id = units[i];
+        if (has_room && i < n) {
+            if (i < in_tiles) {
+                const uint32_t t = i / (uint32_t)L.units;
+                id = (uint64_t)L.tile_list[t] << 8 | (uint64_t)(i - t * (uint32_t)L.units);
+            } else {
+                id = units[i - in_tiles];
+            }
+        }
         uint32_t bits = 0u;
         int eb = 0, ri = 0;
         int64_t row = 0, i1 = 0;
@@ -56,12 +64,16 @@ __device__ __forceinline__ void live_units(const Launch &L, float *s_dyn) {
             const uint32_t tl = (uint32_t)(id >> 8);
             while (ri + 1 < L.n_ranges && (int64_t)tl >= L.rng[ri + 1].tile0) ++ri;
             const RangeDesc &rd = L.rng[ri];
-            const RangeProg &rp = rd.prog;
             const uint32_t lt = tl - (uint32_t)rd.tile0;
             const uint32_t q = lt / (uint32_t)rd.tiles_per_row;
             row = q;
             const int64_t col = lt - q * (uint32_t)rd.tiles_per_row;
             i1 = (col * L.units + (int64_t)(id & 255u)) * kX;   // the unit's first start
+            if (i1 >= rd.n_emit) id = ~0ull;   // a listed tile's unit past the row's last start
+        }
+        if (id != ~0ull) {
+            const RangeDesc &rd = L.rng[ri];
+            const RangeProg &rp = rd.prog;
             const int entry = rd.per_row ? (int)row : 0;
             const bool has_sc = rd.scale != nullptr;
             const float sc = has_sc ? rd.scale[row] : 1.f;

@@ -1046,15 +1046,24 @@ __device__ __forceinline__ void search_tiles(const Launch &L, unsigned char *sme
 }
 
 // The tiles, then (after a screen) the live units of the tiles not searched
-// whole.
+// whole.  A tile takes its CTA 10 to 20 us however few there are, so when their
+// units make no more than two rounds of the launch's half-warps (some 40 tiles
+// of wmax 256) they are searched as units too.
 template <int DT, int G, bool MG, int NT, bool PL>
 __global__ void __launch_bounds__(NT, 512 / NT) search_kernel(const __grid_constant__ Launch L) {
     extern __shared__ __align__(16) unsigned char smem[];
-    search_tiles<DT, G, MG, NT, PL>(L, smem);
+    uint32_t in_tiles = 0;   // units of listed tiles that the half-warps search
+    if constexpr (!PL && NT == kSearchThreads) {
+        if (L.unit_list) {
+            const uint64_t u = (uint64_t)*L.tile_count * (uint32_t)L.units;
+            if (u <= 2ull * gridDim.x * (uint32_t)L.live_halves) in_tiles = (uint32_t)u;
+        }
+    }
+    if (!in_tiles) search_tiles<DT, G, MG, NT, PL>(L, smem);
     if constexpr (!PL && NT == kSearchThreads) {
         if (L.unit_list) {
             __syncthreads();
-            live_units<DT, G, MG>(L, reinterpret_cast<float *>(smem));
+            live_units<DT, G, MG>(L, reinterpret_cast<float *>(smem), in_tiles);
         }
     }
 }
