@@ -67,6 +67,19 @@ __device__ __forceinline__ void pmax1(float &m0, float &m1, float2 sa, uint32_t 
     m1 = fmaxf(m1, packw(sa.y, ka));
 }
 
+// Two adds, or multiplies, one by one.  The pairs of the step-1 groups are no
+// neighbours in memory and their ring turns, so packed arithmetic paid for its
+// operands with moves: plane output of 256 x 262144 samples, widths 1..64, 967
+// us packed and 851 so (1..128: 2243 and 1890; the SKA-like search 13.66 and
+// 13.18 ms).  The step-G groups, whose pairs are loaded as such, keep it (713
+// us for 46 widths; 738 with their products one by one).
+__device__ __forceinline__ float2 add1(float2 a, float2 b) {
+    return make_float2(__fadd_rn(a.x, b.x), __fadd_rn(a.y, b.y));
+}
+__device__ __forceinline__ float2 mul1(float2 a, float b) {
+    return make_float2(__fmul_rn(a.x, b), __fmul_rn(a.y, b));
+}
+
 // Step-1 group, pairs of samples (k, k + 8): B[j] = (B(16t + j), B(16t + j + 8)).
 // The step of width c for pair j is (y[off + c + j], y[off + c + j + 8])
 // (positions relative to 16t), held in ring slot (j + c) & 7: from one width
@@ -101,22 +114,20 @@ __device__ __forceinline__ void eval_fine(float (&cb)[kX], float2 (&B)[8], const
             const int wi = g.widx0 + c;
             const uint32_t ka = 63u - (uint32_t)(wi & 63);
             const float ia = s_inv[wi];
-            const float2 ia2 = make_float2(ia, ia);
             float2 sa[8];
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
-                B[j] = add2(B[j], R[(j + cc) & 7]);
-                sa[j] = mul2(B[j], ia2);
+                B[j] = add1(B[j], R[(j + cc) & 7]);
+                sa[j] = mul1(B[j], ia);
             }
             R[cc].x = R[cc].y;
             R[cc].y = AL ? ynext[kSPad * (c >> 4) + (c & 15)] : yb[sadr(off + c + 16)];
             if (c + 1 < g.count) {
                 const float ib = s_inv[wi + 1];
-                const float2 ib2 = make_float2(ib, ib);
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
-                    B[j] = add2(B[j], R[(j + cc + 1) & 7]);
-                    pmax2(cb[j], cb[j + 8], sa[j], mul2(B[j], ib2), ka);
+                    B[j] = add1(B[j], R[(j + cc + 1) & 7]);
+                    pmax2(cb[j], cb[j + 8], sa[j], mul1(B[j], ib), ka);
                 }
                 R[cc + 1].x = R[cc + 1].y;
                 R[cc + 1].y = AL ? ynext[kSPad * ((c + 1) >> 4) + ((c + 1) & 15)]
@@ -222,11 +233,10 @@ __device__ __forceinline__ void eval_generic(float (&cb)[kX], float2 (&B)[8], co
         const int wi = g.widx0 + c;
         const uint32_t ka = 63u - (uint32_t)(wi & 63);
         const float ia = s_inv[wi];
-        const float2 ia2 = make_float2(ia, ia);
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-            B[j] = add2(B[j], make_float2(sb[sadr(p0 + 2 * j)], sb[sadr(p0 + 2 * j + 1)]));
-            pmax1(cb[2 * j], cb[2 * j + 1], mul2(B[j], ia2), ka);
+            B[j] = add1(B[j], make_float2(sb[sadr(p0 + 2 * j)], sb[sadr(p0 + 2 * j + 1)]));
+            pmax1(cb[2 * j], cb[2 * j + 1], mul1(B[j], ia), ka);
         }
     }
 }
