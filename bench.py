@@ -36,10 +36,12 @@ UNIT = "DM×time samples/s"
 WIDTHS = list(range(1, 17)) + list(range(24, 257, 8))
 THRESHOLD = 7.0
 SAMPLE_TIME_S = 64e-6
-# msd_partial, msd_merge_l1, fold_final, merge_shards, consts, detect
-KERNELS_PER_STEP = 6
+# msd_partial, msd_merge_l1, fold_final, merge_shards, consts, screen, search
+KERNELS_PER_STEP = 7
 PROFILES = os.path.join(ROOT, "profiles")
-DETECT_SRC = os.path.join(ROOT, "paper_1611_09704_gb300", "csrc", "spd_search_kernel.cuh")
+# the kernels of the detect phase: the screen and the search of what it keeps
+DETECT_SRC = [os.path.join(ROOT, "paper_1611_09704_gb300", "csrc", f)
+              for f in ("spd_search_kernel.cuh", "spd_live.cuh", "spd_screen.cu")]
 
 
 def parse():
@@ -86,8 +88,11 @@ def peaks():
 
 
 def detect_source_sha() -> str:
-    with open(DETECT_SRC, "rb") as f:
-        return hashlib.sha256(f.read()).hexdigest()[:16]
+    h = hashlib.sha256()
+    for path in DETECT_SRC:
+        with open(path, "rb") as f:
+            h.update(f.read())
+    return h.hexdigest()[:16]
 
 
 def traffic_file(workload: str) -> str:
@@ -417,7 +422,7 @@ def run_spd(a, rank, world, local):
             "config": workload_config(n_dm, n_samp, world),
             "realtime_factor": n_samp * SAMPLE_TIME_S / (ms_step / 1e3),
             "candidates_per_step": count,
-            "roofline": hbm_roofline("search_kernel (boxcar + SNR + max + threshold)",
+            "roofline": hbm_roofline("screen_kernel + search_kernel (boxcar + SNR + max + threshold)",
                                      det_bytes, det_ms, traffic),
             "issue_roofline": issue_roofline(n, det_ms),
             "step_breakdown_ms": {"msd": msd_ms, "detect": det_ms},
@@ -619,7 +624,7 @@ def run_other(a):
         ms, clocks = timed(step, a.steps, a.warmup, 0)
         count = spd.read_result(res)[0]
         line.update(value=n / (ms / 1e3), ms_per_step=ms, dtype="f32", clocks=clocks,
-                    candidates_per_step=count, gpu_launches=5 * a.steps,
+                    candidates_per_step=count, gpu_launches=4 * a.steps,
                     roofline=hbm_roofline("search step (MSD + search kernel)",
                                           2 * 4 * n + 16 * count, ms,
                                           note="inputs L2-resident (16.8 MB): latency-bound"),
@@ -647,7 +652,11 @@ def run_other(a):
             ctypes.byref(spd.Plane(x, scale=scale).c()), 0, 256), 1), dtype=torch.uint8,
             device=dev)
         for mode, name in ((1, "eq5_as_printed"), (2, "eq5_linear_excess")):
-            dws = torch.empty(1 << 20, dtype=torch.uint8, device=dev)
+            prm, keep = spd.binding._params(widths, THRESHOLD, mode, 0, 256)
+            dws = torch.empty(spd.binding.load().spd_detect_workspace_bytes(
+                ctypes.byref(spd.Plane(x, scale=scale).c()), ctypes.byref(prm)),
+                dtype=torch.uint8, device=dev)
+            del keep
             phases = [lambda: spd.msd(x, 0, 256, out=msd, workspace=mws, scale=scale),
                       lambda mode=mode: spd.detect(x, msd, widths, THRESHOLD, out.shape[0], mode,
                                                    0, 256, out=out, result=res, workspace=dws,
@@ -664,8 +673,8 @@ def run_other(a):
         bd = main_["step_breakdown_ms"]
         line.update(value=main_["value"], ms_per_step=main_["ms_per_step"], dtype=a.dtype,
                     clocks=main_["clocks"], candidates_per_step=main_["candidates"],
-                    gpu_launches=8 * a.steps, modes=modes,
-                    roofline=hbm_roofline("search_kernel (boxcar + SNR + max + threshold)",
+                    gpu_launches=7 * a.steps, modes=modes,
+                    roofline=hbm_roofline("screen_kernel + search_kernel (boxcar + SNR + max + threshold)",
                                           in_bytes + 16 * main_["candidates"], bd["detect"],
                                           recorded_traffic(n, main_["candidates"],
                                                            f"precision_{a.dtype}")),
@@ -700,7 +709,7 @@ def run_other(a):
         cnt = spd.read_result(bs.result)[0]
         in_bytes = n * 4
         line.update(value=n / (ms / 1e3), ms_per_step=ms, dtype="f32", clocks=clocks,
-                    candidates_per_step=cnt, gpu_launches=(5 * len(specs) + 1) * a.steps,
+                    candidates_per_step=cnt, gpu_launches=(2 * len(specs) + 2) * a.steps,
                     tuning=tune, realtime_factor=dur / (ms / 1e3),
                     roofline=hbm_roofline("batched step (per-range MSD + one search-kernel "
                                           "launch), one graph replay", 2 * in_bytes + 16 * cnt,
@@ -741,7 +750,7 @@ def run_other(a):
         ms2, _ = timed(step2, max(3, a.steps // 4), 3, 0)
         cnt2 = spd.read_result(res)[0]
         line.update(value=n / (ms / 1e3), ms_per_step=ms, dtype="f32", clocks=clocks,
-                    candidates_per_step=cnt, gpu_launches=(4 + 5 * len(levels)) * a.steps,
+                    candidates_per_step=cnt, gpu_launches=(5 + 2 * len(levels)) * a.steps,
                     plain_search={"widths": "1..512", "ms_per_step": ms2, "value": n / (ms2 / 1e3),
                                   "candidates": cnt2},
                     roofline=hbm_roofline("decimated step (level planes, per-level MSD, one "
@@ -909,7 +918,9 @@ def run_serving(a, spd, synth, line, dev):
                                       note="host-driven pass timed by wall clock: bounded by "
                                            "the scheduler and host link, not one kernel"),
                 candidates_per_step=sat["candidates"],
-                gpu_launches=n_chunks * 4 + len(beams) * 4,   # push: 4 kernels; reset+flush: 4
+                # push: MSD, merge, screen, search and the halo out (and in,
+                # but for a beam's first); reset and flush: 5
+                gpu_launches=n_chunks * 6 + len(beams) * 4,
                 saturated=dict(sat, max_inflight=inflight_sat),
                 realtime=dict(rt, compress=a.compress, max_inflight=srv.scheduler.max_inflight),
                 realtime_factor=sat["samples"] / n_dm * SAMPLE_TIME_S / sat["span_s"],

@@ -301,18 +301,22 @@ spd_status spd_threshold_plane(float *snr, uint16_t *width, int64_t n_dm, int64_
  *     capacity is 0); result_dev->count is set to the exact number of
  *     clusters (the call zeroes it first), and only the first `capacity`
  *     records are written.
- * One warp scans one row.  Errors: SPD_ERR_INVALID_ARG, SPD_ERR_CUDA. */
+ * A row is scanned in segments at once; a cluster belongs to the segment it
+ * starts in.  Errors: SPD_ERR_INVALID_ARG, SPD_ERR_CUDA. */
 spd_status spd_cluster_rows(const float *snr, const uint16_t *width, int64_t n_dm,
                             int64_t n_samp, int64_t stride, float threshold, int32_t max_gap,
                             spd_cluster *out, int64_t capacity, spd_result *result_dev,
                             void *stream);
 
-/* Bytes of device workspace spd_detect / spd_search need. */
+/* Bytes of device workspace spd_detect / spd_search need.  The last piece holds
+ * the lists of the screen, which finds the tiles and units of 16 starts that
+ * can hold a candidate; a workspace too small for that piece alone is accepted,
+ * and every tile is searched: the same records, later. */
 size_t spd_detect_workspace_bytes(const spd_plane *plane, const spd_search_params *params);
 size_t spd_search_workspace_bytes(const spd_plane *plane, const spd_search_params *params);
 
-/* Steps (b)+(c)+(d) fused in one kernel given the MSD (msd_dev as for
- * spd_boxcar_snr): boxcars, SNR, max over widths and thresholding happen in
+/* Steps (b)+(c)+(d) fused given the MSD (msd_dev as for spd_boxcar_snr), over
+ * what a screen of the plane keeps: boxcars, SNR, max over widths and thresholding happen in
  * registers and shared memory; only candidate records leave the SM.  The
  * candidate set equals thresholding spd_boxcar_snr's output.
  * Errors: as spd_boxcar_snr, plus result semantics as spd_threshold_candidates. */
@@ -324,7 +328,8 @@ spd_status spd_detect(const spd_plane *plane, const spd_search_params *params,
 /* The whole path: spd_msd (a) then spd_detect (b, c, d) on one stream.
  *   msd_out_dev: optional device array (1 or n_dm entries) receiving the MSD;
  *     NULL keeps it inside the workspace.
- * The plane is read twice from HBM: once for the MSD, once for the search,
+ * The plane is read twice from HBM, once for the MSD and once for the screen,
+ * and what the screen keeps a third time by the search,
  * because no SNR is known before the dataset's sigma is (Sec. 2.1 -> 2.3). */
 spd_status spd_search(const spd_plane *plane, const spd_search_params *params,
                       spd_candidate *out, int64_t capacity, spd_result *result_dev,
@@ -390,8 +395,8 @@ size_t spd_search_batched_workspace_bytes(const spd_range *ranges, int32_t n_ran
                                           const spd_tuning *tuning);
 
 /* The whole path over up to SPD_MAX_RANGES DM ranges of uneven length, width
- * set and decimation: per range the MSD (a) and its constants, then ONE
- * persistent detect launch (b, c, d) whose CTAs walk the tiles of all ranges
+ * set and decimation: the MSD (a) and the constants of every range, then ONE
+ * screen and ONE persistent search launch (b, c, d) over the tiles of all ranges
  * -- per launch, ranges whose width lists step by the same G (8, 16 or 1) and
  * that share storage type and row alignment.  Every call is a fixed sequence of
  * asynchronous launches with no host synchronisation and no allocation, so it

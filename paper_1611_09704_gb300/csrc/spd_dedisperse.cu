@@ -89,7 +89,7 @@ __device__ __forceinline__ void cp_async_wait_all() {
 // registers of sums per thread).  256 channels x 256 trials x 2^18 outputs
 // FP32: 3.40 ms with one word per output, trial and channel, 4-byte copies and
 // 2 outputs per thread (5.9 instructions per add); 2.97 ms with sums of pairs
-// and 4 outputs; 2.41 ms with the copies' addresses prepared once per channel
+// and 4 outputs; 2.44 ms with the copies' addresses prepared once per channel
 // and whole blocks of the sums formed without bound checks (2.8 per add).  200
 // x 117 x 60001 FP16: 583 -> 300 us (16-bit windows staged as they are).
 // Trials too far apart to share a window, 200 x 32 x 16000: 0.51 -> 0.14 ms

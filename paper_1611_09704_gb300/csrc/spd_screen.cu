@@ -5,7 +5,7 @@
 // every tile: centred samples, prefixes and window sums in shared memory, the
 // table of prefix maxima, a bound per width group.  The screen does only what
 // is needed to know which units of 16 starts can hold a candidate at all: it
-// reads every sample once, straight into registers, keeps five numbers per
+// reads every sample once, through a ring of each warp's own, keeps five numbers per
 // block of 16, and makes one test per class of widths.  Tiles with many units
 // that pass are listed whole for the search kernel, the units of the others
 // one by one for its half-warps (spd_live.cuh).

@@ -1,7 +1,8 @@
 // spd_search_kernel.cuh -- the candidate search: steps (b), (c) and (d) fused
 // (boxcar filters, SNR with the max over widths and the winning width, and
 // thresholding with compaction; Sec. 2.3-2.4, Algorithm 1) over one or more
-// DM ranges in one persistent launch.
+// DM ranges in one persistent launch.  After a screen (spd_screen.cu) only the
+// tiles and units that it lists are searched, the units by live_units.
 //
 // CTAs of 256 (or 128) threads walk tiles of 16 U consecutive start samples
 // of one DM row, U = the threads less the halo's blocks, so that every thread
@@ -35,8 +36,8 @@
 //
 // Evaluation follows Algorithm 1: a group's running sums start at B_off (the
 // sum of whole blocks plus the difference of in-block prefixes) and grow by
-// one sample (step 1) or one window sum (step G) per width, two samples per
-// packed f32x2 add and multiply.  Each SNR is packed with a code (63 minus the
+// one sample (step 1) or one window sum (step G) per width, the latter two
+// samples per packed f32x2 add and multiply.  Each SNR is packed with a code (63 minus the
 // eval index within its block of 64) in its low 6 mantissa bits before a
 // float max, so one max keeps value and width; among SNRs equal to 2^-17
 // relative the smallest width wins -- the strict ">" of Algorithm 1 at that
