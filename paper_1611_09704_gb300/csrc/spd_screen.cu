@@ -131,20 +131,26 @@ __host__ __device__ inline int screen_warp_bytes(int esz, int rows) {
 // NaN bound, too).  Windows past the row end do not exist for it.
 //
 // kTop: the widest class of the launch (3, 5, 6 or 9).  Widths up to 512 have
-// their own form with fixed reads: the four ranges of a batched search (to 64,
-// 128, 256 and 512) 1.24 ms through the loop for any width, 1.17 ms so.
+// their own forms, with fixed reads and, as they reach 32 blocks at most, a lag
+// of one round and a ring of two.  kScaled: some range of the launch has a
+// scale (a range without one then takes 1 and 0).  Both are arguments of the
+// template because a branch between the scaled and the plain samples moved all
+// of them at its end: 4096 x 524288 FP32 1.33 ms with the branch and the ring's
+// sizes read, 1.20 with these fixed, 1.17 without the branch; the four ranges
+// of a batched search (to 64, 128, 256 and 512) 1.17, 1.06 and 1.03 ms; 2048 x
+// 524288 FP16 with a scale 0.69, 0.63 and 0.62 ms.
 //
 // Bound by the plane's one read in FP32: 4096 x 524288 samples (8.6 GB) in
-// 1.32 ms, 6.5 TB/s of the 6.8 a plain copy reaches; in FP16 by instruction
-// issue (2048 x 524288 in 0.69 ms, 3.1 TB/s).  Before, the search kernel took
-// 10.3 and 4.9 ms over every tile of the same planes.  A first form of the
+// 1.17 ms, 7.3 TB/s (a plain copy, half of it writes, reaches 6.8); in FP16 by
+// instruction issue (3.5 TB/s).  Before, the search kernel took 10.3 and 4.9 ms
+// over every tile of the same planes.  A first form of the
 // screen, with a CTA over four tiles, a lane's 64 bytes loaded to registers
 // and CTA barriers between the prefix passes, took 2.14 ms (the loads touch 16
 // lines each); the copies here, with a test written class by class, 1.75 ms
-// (407 instructions per warp and round against 300 as it stands).  72
+// (407 instructions per warp and round).  72
 // registers and 7.9 KB leave 7 CTAs of 4 warps per SM, two rounds in flight in
 // each warp: 112 KB per SM.
-template <int DT, int kTop>
+template <int DT, int kTop, bool kScaled>
 __global__ void __launch_bounds__(kScrThreads, 7)
     screen_kernel(const __grid_constant__ ScreenArgs A) {
     using T = typename Elem<DT>::T;
@@ -157,7 +163,9 @@ __global__ void __launch_bounds__(kScrThreads, 7)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t tile = blockIdx.x * kScrWarps + warp;
     if (tile >= A.n_tiles) return;              // the whole warp; no barrier spans warps
-    const int rows = A.ring + A.mirror;         // rounds stored, the mirrored ones included
+    // widths up to 512 reach 32 blocks at most: a lag of one round, a ring of two
+    const int ring = kTop > 6 ? A.ring : 2, mirror = kTop > 6 ? A.mirror : 1;
+    const int rows = ring + mirror;             // rounds stored, the mirrored ones included
     unsigned char *buf = s_raw + warp * screen_warp_bytes(kEsz, rows);
     float2 *s_e = reinterpret_cast<float2 *>(buf + kScrBufs * kBuf);   // half-block energies
     float *s_x = reinterpret_cast<float *>(s_e + rows * 32);           // largest C
@@ -180,7 +188,7 @@ __global__ void __launch_bounds__(kScrThreads, 7)
     const int rounds = (nb + 31) >> 5;
     const int have = (int)min((int64_t)rounds * 512, rd.n_samp - t0);   // positions inside the row
     const T *rowp = static_cast<const T *>(rd.data) + (int64_t)row * rd.stride + t0;
-    const bool has_sc = rd.scale != nullptr;
+    const bool has_sc = kScaled && rd.scale != nullptr;
     const float sc = has_sc ? rd.scale[row] : 1.f;
     const float of = (has_sc && rd.offset) ? rd.offset[row] : 0.f;
     const float2 mu = rd.mu_tab[entry];
@@ -296,8 +304,8 @@ __global__ void __launch_bounds__(kScrThreads, 7)
         total += __popc(bal);
     };
 
-    const int lag = (reach + 31) >> 5;   // rounds from a unit to the last block it reads
-    const int ring = A.ring;
+    // rounds from a unit to the last block it reads
+    const int lag = kTop > 6 ? (reach + 31) >> 5 : 1;
     float run = 0.f, mag = 0.f;
     uint32_t at = 0;                     // the buffer of round r, and of round r + 2
     uint32_t at2 = 2 * kBuf;
@@ -313,13 +321,14 @@ __global__ void __launch_bounds__(kScrThreads, 7)
         stage(r + 2, at2);
         at = at == 2 * kBuf ? 0 : at + kBuf;
         at2 = at2 == 2 * kBuf ? 0 : at2 + kBuf;
-        if (has_sc) {
+        if constexpr (kScaled) {
             const float2 s2 = make_float2(sc, sc), o2 = make_float2(of, of);
 #pragma unroll
-            for (int q = 0; q < 8; ++q) v[q] = fma2(s2, v[q], o2);
-        }
+            for (int q = 0; q < 8; ++q) v[q] = add2(add2(fma2(s2, v[q], o2), mh), ml);
+        } else {
 #pragma unroll
-        for (int q = 0; q < 8; ++q) v[q] = add2(add2(v[q], mh), ml);
+            for (int q = 0; q < 8; ++q) v[q] = add2(add2(v[q], mh), ml);
+        }
         float sum = 0.f, hi = 0.f, lo = 0.f;
         float2 e0 = make_float2(0.f, 0.f), e1 = e0;
         if (512 * r + 512 <= have) {          // warp-uniform
@@ -377,14 +386,16 @@ __global__ void __launch_bounds__(kScrThreads, 7)
             if (kTop > 5) m8 = fmaxf(m4, __shfl_xor_sync(0xffffffffu, m4, 4));
         }
         const int rr = r & (ring - 1);
-        for (int k = rr; k < rows; k += ring) {   // the round, and its mirror
+        auto keep = [&](int k) {
             const int slot = 32 * k + lane;
             s_x[slot] = mx;
             s_n[slot] = mn;
             s_e[slot] = en;
             if (kTop > 3) s_q4[slot >> 2] = m4;   // the same value from each of the lanes
             if (kTop > 5) s_q8[slot >> 3] = m8;
-        }
+        };
+        keep(rr);
+        if (rr < mirror) keep(rr + ring);
         // the prefixes are off by some 30 roundings of the tile's largest
         // partial sum so far at most (in-block 16, the scan, the running
         // total, and their uses): the margin is six times that
@@ -424,10 +435,14 @@ __global__ void __launch_bounds__(kScrThreads, 7)
     }
 }
 
-template <int DT> void (*screen_of(int top))(const ScreenArgs) {
-    return top <= 3   ? screen_kernel<DT, 3>
-           : top <= 5 ? screen_kernel<DT, 5>
-           : top <= 6 ? screen_kernel<DT, 6> : screen_kernel<DT, 9>;
+template <int DT, bool kScaled> void (*screen_of(int top))(const ScreenArgs) {
+    return top <= 3   ? screen_kernel<DT, 3, kScaled>
+           : top <= 5 ? screen_kernel<DT, 5, kScaled>
+           : top <= 6 ? screen_kernel<DT, 6, kScaled> : screen_kernel<DT, 9, kScaled>;
+}
+template <bool kScaled> void (*screen_of(int dtype, int top))(const ScreenArgs) {
+    return dtype == SPD_F32 ? screen_of<SPD_F32, kScaled>(top)
+           : dtype == SPD_F16 ? screen_of<SPD_F16, kScaled>(top) : screen_of<SPD_BF16, kScaled>(top);
 }
 
 }  // namespace
@@ -435,6 +450,7 @@ template <int DT> void (*screen_of(int top))(const ScreenArgs) {
 cudaError_t launch_screen(const Launch &L, const ScreenLists &S, int dtype, cudaStream_t s) {
     static thread_local ScreenArgs A;
     int lag = 1, widest = 0;
+    bool scaled = false;
     for (int r = 0; r < L.n_ranges; ++r) {
         const RangeDesc &rd = L.rng[r];
         ScreenRange &q = A.rng[r];
@@ -443,6 +459,7 @@ cudaError_t launch_screen(const Launch &L, const ScreenLists &S, int dtype, cuda
         q.n_samp = rd.n_samp;
         q.n_emit = rd.n_emit;
         q.scale = rd.scale;
+        scaled |= rd.scale != nullptr;
         q.offset = rd.offset;
         q.mu_tab = rd.mu_tab;
         q.flags = rd.flags;
@@ -481,8 +498,7 @@ cudaError_t launch_screen(const Launch &L, const ScreenLists &S, int dtype, cuda
     if (L.n_tiles <= 0) return cudaSuccess;
     const size_t smem =
         (size_t)kScrWarps * screen_warp_bytes((int)elem_bytes(dtype), A.ring + A.mirror);
-    auto k = dtype == SPD_F32 ? screen_of<SPD_F32>(widest)
-             : dtype == SPD_F16 ? screen_of<SPD_F16>(widest) : screen_of<SPD_BF16>(widest);
+    auto k = scaled ? screen_of<true>(dtype, widest) : screen_of<false>(dtype, widest);
     if (smem > 48 * 1024) {   // wide lists
         const cudaError_t e =
             cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
