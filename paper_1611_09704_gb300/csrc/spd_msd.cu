@@ -13,6 +13,7 @@
 #include "spd_internal.cuh"
 
 #include <math.h>
+#include <type_traits>
 
 namespace spd {
 
@@ -683,9 +684,10 @@ __device__ __forceinline__ float block_sum(const float *s_y, int b) {
 // partial.  The sd does not depend on the centring.
 //
 // Bound by latency at 20 warps per SM (96 registers; six CTAs of 80 spill and
-// take 757 us): 2048 x 524288 FP16, Nmax 256, in 700 us, of which the one read
+// take 757 us): 2048 x 524288 FP16, Nmax 256, in 684 us, of which the one read
 // needs 317.  With the padded addresses formed for every load and 64-bit counts
-// compared every 16 starts it took 864 us (20 instructions per sample, now 14).
+// compared every 16 starts it took 864 us (20 instructions per sample, now 14),
+// with the choice between aligned and other windows inside the slide 700.
 template <int DT>
 __global__ void __launch_bounds__(kNmaxThreads, 5) nmax_partial_kernel(const NmaxArgs a) {
     using T = typename Elem<DT>::T;
@@ -806,15 +808,17 @@ __global__ void __launch_bounds__(kNmaxThreads, 5) nmax_partial_kernel(const Nma
         const int64_t nv64 = a.n_samp - nmax - (t0 + 16 * b0) + 1;
         const int nvalid = nv64 < 0 ? 0 : nv64 < kNmaxPer ? (int)nv64 : kNmaxPer;
         // the unit's 16 samples and the 16 that enter the window as it slides;
-        // d slides by hi - lo per start (the differences as f32x2 pairs)
-        auto slide = [&](int c, float2 (&bw)[8]) {   // bw[k] = d at unit starts 2k, 2k + 1
+        // d slides by hi - lo per start (the differences as f32x2 pairs).
+        // whole: nmax is a multiple of 16, so what enters lies in 128-bit words;
+        // in: from the thread's run to it
+        auto slide = [&](auto whole, int c, int in, float2 (&bw)[8]) {   // bw[k] = d at unit starts 2k, 2k + 1
             const float *lp = own + 16 * c;
-            const float *hp = own + enter[c];
+            const float *hp = own + in;
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 const float4 lo = *reinterpret_cast<const float4 *>(lp + 4 * q);
                 float4 hi;
-                if ((nmax & 15) == 0) {
+                if constexpr (decltype(whole)::value) {
                     hi = *reinterpret_cast<const float4 *>(hp + 4 * q);
                 } else {
                     const int p = kNmaxPer * tid + 16 * c + 4 * q + nmax;
@@ -831,24 +835,30 @@ __global__ void __launch_bounds__(kNmaxThreads, 5) nmax_partial_kernel(const Nma
                 Bd = bw[2 * q + 1].y + db.y;
             }
         };
-        if (nvalid == kNmaxPer) {
+        auto full = [&](auto whole) {
 #pragma unroll
             for (int c = 0; c < kNmaxPer / 16; ++c) {
                 float2 bw[8];
-                slide(c, bw);
+                slide(whole, c, enter[c], bw);
 #pragma unroll
                 for (int k = 0; k < 8; ++k) {
                     Td = __fadd2_rn(Td, bw[k]);
                     Sd = __ffma2_rn(bw[k], bw[k], Sd);
                 }
             }
+        };
+        if (nvalid == kNmaxPer) {
+            if ((nmax & 15) == 0) full(std::true_type{});
+            else full(std::false_type{});
             nrun = kNmaxPer;
         } else {   // near the row end: the starts with full windows
 #pragma unroll 1
             for (int c = 0; 16 * c < nvalid; ++c) {
                 const int nv = nvalid - 16 * c;
                 float2 bw[8];
-                slide(c, bw);
+                const int in = npad(16 * c + nmax);
+                if ((nmax & 15) == 0) slide(std::true_type{}, c, in, bw);
+                else slide(std::false_type{}, c, in, bw);
 #pragma unroll
                 for (int k = 0; k < 8; ++k) {
                     const float2 dm = make_float2(2 * k < nv ? bw[k].x : 0.f,
