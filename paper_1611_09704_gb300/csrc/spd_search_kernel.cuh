@@ -429,7 +429,7 @@ __device__ __forceinline__ void search_tiles(const Launch &L, unsigned char *sme
         if (PL) return tile + 1 >= s_ntiles;
         return (((uint32_t)tile + 1u) & (uint32_t)(s_chunk - 1)) == 0u || tile + 1 == s_ntiles;
     };
-    __shared__ long long s_next;                // first tile of the next chunk, or -1
+    __shared__ long long s_next;                // first tile of the next chunk, or -1 (not PL)
     __shared__ unsigned s_claim;                // thread 0's claim for the chunk after this one
     unsigned claim = 0;                         // thread 0, until it parks it in s_claim
     bool claimed = !PL && tid == 0;
@@ -503,8 +503,8 @@ __device__ __forceinline__ void search_tiles(const Launch &L, unsigned char *sme
                 const int64_t nc = (int64_t)gridDim.x + (int64_t)v;
                 if (nc < n_chunks) nt = nc * ch;
                 else if ((int64_t)v == n_chunks - 1) atomicExch(counter(), 0u);   // the last claim
+                s_next = nt;
             }
-            s_next = nt;
         }
         if (tma && nt >= 0) issue(nt == tile + 1 ? advance(pos) : pos_of(nt));
     };
@@ -574,7 +574,12 @@ __device__ __forceinline__ void search_tiles(const Launch &L, unsigned char *sme
                 ++tile;
                 pos = advance(pos);
             } else {
-                const int64_t nt = s_next;   // written before the last barrier
+                // a PL run ends with its last tile, which every thread sees for
+                // itself: PL has no barrier between issue_next and this place
+                // (a warp without units comes here at once) that would publish
+                // s_next
+                if (PL) break;
+                const int64_t nt = s_next;   // written before barrier (C)
                 if (nt < 0) break;
                 tile = nt;
                 pos = pos_of(tile);
