@@ -506,7 +506,8 @@ __device__ __forceinline__ void search_tiles(const Launch &L, unsigned char *sme
                 s_next = nt;
             }
         }
-        if (tma && nt >= 0) issue(nt == tile + 1 ? advance(pos) : pos_of(nt));
+        // (neighbours in a list are no neighbours in the plane)
+        if (tma && nt >= 0) issue(!list && nt == tile + 1 ? advance(pos) : pos_of(nt));
     };
 
     int64_t key = -1;                       // (range, scope entry) of the constants loaded
