@@ -502,7 +502,8 @@ def search(x, widths, threshold, capacity, sigma_mode=SIGMA_SQRTN, scope=MSD_GLO
 def debug_set_copy_wait(limit_ns=2_000_000_000, extra_bytes=0):
     """spd_debug_set_copy_wait (test aid): bound of the fused kernel's waits
     for tile copies, and bytes expected beyond each copy (> 0 makes every wait
-    run out); the defaults restore normal operation."""
+    run out; 16: those of every tile, more: those of the tiles that a screen
+    lists); the defaults restore normal operation."""
     _check(load().spd_debug_set_copy_wait(int(limit_ns), int(extra_bytes)),
            "spd_debug_set_copy_wait")
 

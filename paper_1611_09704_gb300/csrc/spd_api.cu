@@ -348,7 +348,8 @@ spd_status range_consts(const spd_plane *p, const RangeProg &prog, const spd_msd
 }
 
 // Bound of a wait for a bulk copy, and bytes expected beyond each copy (a
-// test aid that makes the waits run out); set by spd_debug_set_copy_wait.
+// test aid that makes the waits run out; 16: over every tile, without a screen);
+// set by spd_debug_set_copy_wait.
 thread_local uint64_t g_wait_ns = 2000000000ull;
 thread_local uint32_t g_extra_tx = 0;
 
@@ -360,8 +361,8 @@ thread_local uint32_t g_extra_tx = 0;
 // With `lists` (the ranges carrying the screen's tables) the launch is two:
 // the screen, then the search kernel over the tiles it lists and the live
 // units of the rest.  Not with 128-thread tiles (the lists are sized for 256), nor
-// while the test aid makes the search kernel's copies run out: then every
-// tile is searched.
+// while the test aid makes the copies of every tile run out: then every tile is
+// searched.
 spd_status run_launch(const RangeDesc *rd, int n, int dtype, spd_candidate *out, int64_t cap,
                       spd_result *result, float *snr_out, uint16_t *width_out,
                       int64_t out_stride, int ctas_per_sm, cudaStream_t st, int threads = 0,
@@ -423,7 +424,7 @@ spd_status run_launch(const RangeDesc *rd, int n, int dtype, spd_candidate *out,
     L.units = units;
     const size_t smem = search_smem_bytes(L.R, raw, max_eval, kmax, G);
     if (smem > 227 * 1024) return SPD_ERR_UNSUPPORTED;
-    const bool screen = lists && lists->ctl && !snr_out && nt == kSearchThreads && !g_extra_tx &&
+    const bool screen = lists && lists->ctl && !snr_out && nt == kSearchThreads && g_extra_tx != 16 &&
                         tiles <= lists->tile_cap && tiles < (int64_t)1 << 24;
     size_t lsmem = smem;
     if (screen && tiles > 0) {

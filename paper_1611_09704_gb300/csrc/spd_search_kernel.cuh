@@ -360,8 +360,10 @@ struct TilePos {
     int64_t row, col;
 };
 
+// False (for the whole CTA) when a bulk copy timed out: it may still land in
+// the shared memory, whose barrier counts it, so neither is to be used again.
 template <int DT, int G, bool MG, int NT, bool PL>
-__device__ __forceinline__ void search_tiles(const Launch &L, unsigned char *smem) {
+__device__ __forceinline__ bool search_tiles(const Launch &L, unsigned char *smem) {
     constexpr int kThreads = NT;
     // units of 16 starts per tile: NT less the halo blocks when the whole
     // window then fits one block per thread (one staging round), else NT
@@ -422,7 +424,7 @@ __device__ __forceinline__ void search_tiles(const Launch &L, unsigned char *sme
         s_chunk = L.chunk;
     }
     __syncthreads();
-    if (list && tile >= s_ntiles) return;   // more CTAs than listed tiles
+    if (list && tile >= s_ntiles) return true;   // more CTAs than listed tiles
     // chunks are aligned and a power of two long: a tile is its chunk's last
     // when the next one starts a chunk
     auto chunk_ends = [&]() {
@@ -605,7 +607,7 @@ __device__ __forceinline__ void search_tiles(const Launch &L, unsigned char *sme
                     if (L.result) atomicExch(&L.result->status, (int)SPD_ERR_TIMEOUT);
                     mbar_wait(s_bar, (uint32_t)(k & 1), L.wait_ns);
                 }
-                return;
+                return false;
             }
         } else {
             __syncthreads();
@@ -1054,12 +1056,14 @@ __device__ __forceinline__ void search_tiles(const Launch &L, unsigned char *sme
         pwtot = __reduce_add_sync(0xffffffffu, __popc(mask));
         if (lane == 0) s_wsum[warp] = pwtot;
     }
-    if (PL) return;
+    if (PL) return true;
     // the last tile's records
     __syncthreads();
     if (tid == kAtomicThread) publish(reserve());
+    if (tma && tid == 0) mbar_inval(s_bar);   // no copy in flight: its place may be used
     __syncthreads();
     flush();
+    return true;
 }
 
 // The tiles, then (after a screen) the live units of the tiles not searched
@@ -1076,7 +1080,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) search_kernel(const __grid_const
             if (u <= 2ull * gridDim.x * (uint32_t)L.live_halves) in_tiles = (uint32_t)u;
         }
     }
-    if (!in_tiles) search_tiles<DT, G, MG, NT, PL>(L, smem);
+    if (!in_tiles && !search_tiles<DT, G, MG, NT, PL>(L, smem)) return;
     if constexpr (!PL && NT == kSearchThreads) {
         if (L.unit_list) {
             __syncthreads();
