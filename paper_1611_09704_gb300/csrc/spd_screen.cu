@@ -294,10 +294,11 @@ __global__ void __launch_bounds__(kScrThreads, 7)
             }
         }
         // a prefix that is not finite (a sample before the unit that is not)
-        // rules nothing out
+        // rules nothing out, nor does an energy: a maximum of two would drop a
+        // NaN, so each is tested
         bool live = all | !(fabsf(base) < kInf) | !(m + base < 0.f);
-        live |= !(fmaxf(ha, hb) < h0);
-        live |= !(fmaxf(x0, x1) - g1 + base < 0.f) & !(fmaxf(ha + eb.x, ea.y + hc) < h1);
+        live |= !(ha < h0) | !(hb < h0);
+        live |= !(fmaxf(x0, x1) - g1 + base < 0.f) & (!(ha + eb.x < h1) | !(ea.y + hc < h1));
         live &= 32 * rt + lane < nu;
         const uint32_t bal = __ballot_sync(0xffffffffu, live);
         if (lane == rt) words = bal;
