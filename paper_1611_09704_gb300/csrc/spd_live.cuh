@@ -178,7 +178,7 @@ __device__ __forceinline__ void live_units(const Launch &L, float *s_dyn, uint32
                 if (s_pq[1 + ((14 + end) >> 4)] * 1.000008f * gt.y < lim2) break;
                 float rmax = -INFINITY;
                 for (int b = (g.off + d) >> 4; b <= (15 + end) >> 4; ++b) rmax = fmaxf(rmax, s_mx[b]);
-                if (fmaxf(rmax + cslack, 0.f) * gt.x < lim_lo) continue;
+                if (fmax_nan(rmax + cslack, 0.f) * gt.x < lim_lo) continue;   // NaN never prunes
                 if (MG && (g.widx0 >> 6) != cur) {
                     if (cur >= 0 && trunc17(cb) >= trunc17(ob)) {
                         ob = cb;
@@ -204,7 +204,7 @@ __device__ __forceinline__ void live_units(const Launch &L, float *s_dyn, uint32
                 if (g.off && (g.off & 15) == 0) {
                     const int o = g.off >> 4;
                     float D;
-                    if (lastO >= o && lastO - o <= 16 && lastD > -INFINITY) {
+                    if (lastO >= o && lastO - o <= 16 && fabsf(lastD) < INFINITY) {
                         D = lastD;
                         for (int b = o; b < lastO; ++b) D = __fsub_rn(D, s_bs[b]);
                     } else {

@@ -880,7 +880,7 @@ __device__ __forceinline__ bool search_tiles(const Launch &L, unsigned char *sme
                 }
                 // prefix bound, with the margin for the rounding of the FP32
                 // prefix; a non-positive bound caps every SNR at 0; NaN stays NaN
-                const float pbound = fmaxf(rmax + cslack, 0.f) * __int_as_float(gb.z);
+                const float pbound = fmax_nan(rmax + cslack, 0.f) * __int_as_float(gb.z);
                 // energy bound (squared); the prefix of energies is non-negative
                 // and rounds by a few ulp of its larger end.  The factor covers
                 // this group and all narrower ones, whose windows lie in the
@@ -888,7 +888,8 @@ __device__ __forceinline__ bool search_tiles(const Launch &L, unsigned char *sme
                 const float ebound2 =
                     fmaf(s_pq[tid + gb.x], 1.000008f, -pq0) * __int_as_float(gb.w);
                 if (ebound2 < lim2) break;
-                // NaN bounds (windows past the row end) never prune
+                // NaN bounds (windows past the row end, or all that follows a
+                // sample of the tile that is not finite) never prune
                 if (pbound < lim_lo) continue;
             }
             Group g;
@@ -923,9 +924,9 @@ __device__ __forceinline__ bool search_tiles(const Launch &L, unsigned char *sme
                     const int o = g.off >> 4;
                     float D;
                     // widest group first: take off the blocks between.  Not
-                    // from a sum that met the row end (-inf): the blocks of
-                    // this group may all lie inside the row
-                    if (lastO >= o && lastO - o <= 16 && lastD > -INFINITY) {
+                    // from a sum that met the row end (-inf) or a sample that
+                    // is not finite: the blocks of this group may avoid it
+                    if (lastO >= o && lastO - o <= 16 && fabsf(lastD) < INFINITY) {
                         D = lastD;
                         for (int b = o; b < lastO; ++b) D = __fsub_rn(D, s_bs[tid + b]);
                     } else {

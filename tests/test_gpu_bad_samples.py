@@ -13,9 +13,7 @@ import synth
 pytestmark = pytest.mark.gpu
 
 DEV = "cuda:0"
-# the sample lies close to the row end: fewer units follow it than make a tile
-# worth searching whole
-N, AT, THR = 2190, 2000, 6.0
+AT, THR = 2000, 6.0
 LISTS = {"8": list(range(1, 9)), "32": list(range(1, 33)), "8-step": [1, 2, 8, 16, 24, 32, 40],
          "far": [1, 2, 3, 20, 900]}
 
@@ -28,13 +26,14 @@ def spd():
     return m
 
 
-def _rows(value):
+def _rows(value, n):
     """(rows with the sample, the sample's place in each, clean rows)"""
-    x = synth.noise_plane(16 * 15, N, device=DEV, seed=7).clamp_(-3, 3)
+    x = synth.noise_plane(16 * 15, n, device=DEV, seed=7).clamp_(-3, 3)
     place = AT + torch.arange(240, device=DEV) // 15
     dist = 1 + torch.arange(240, device=DEV) % 15
     r = torch.arange(240, device=DEV)
     x[r, place - dist] = 12.0
+    x[r, place + 40 + dist] = 12.0
     clean = x.clone()
     x[r, place] = value
     return x, place.cpu().numpy(), clean
@@ -43,6 +42,7 @@ def _rows(value):
 def _expected(x, place, msd, widths, starts):
     """Best SNR of each row's starts over the windows inside the row without the sample."""
     y = x.double().cpu().numpy() - msd["mean"][0]
+    n = x.shape[1]
     best = np.full((x.shape[0], len(starts)), -np.inf)
     for r, bad in enumerate(place):
         v = y[r].copy()
@@ -51,14 +51,14 @@ def _expected(x, place, msd, widths, starts):
         for w in widths:
             for k, d in enumerate(starts):
                 s = bad + d
-                if s + w <= N and not s <= bad < s + w:
+                if s + w <= n and not s <= bad < s + w:
                     best[r, k] = max(best[r, k], (c[s + w] - c[s]) / np.sqrt(w) / msd["sd"][0])
     return best
 
 
-def _check(spd, value, name, starts):
+def _check(spd, value, name, starts, n):
     widths = LISTS[name]
-    x, place, clean = _rows(value)
+    x, place, clean = _rows(value, n)
     msd = spd.msd(clean)
     best = _expected(x, place, spd.msd_to_numpy(msd), widths, starts)
     assert (best >= THR).any(axis=1).any()
@@ -70,7 +70,7 @@ def _check(spd, value, name, starts):
         out, res = spd.detect(x, msd, widths, THR, 1 << 20, workspace=ws)
         count, status = spd.read_result(res)
         assert status == 0
-        got = np.zeros((x.shape[0], N), dtype=bool)
+        got = np.zeros((x.shape[0], n), dtype=bool)
         rec = spd.candidates_to_numpy(out, count)
         got[rec["dm"], rec["sample"]] = True
         have = np.stack([got[r, place[r] + np.asarray(starts)] for r in range(x.shape[0])])
@@ -81,4 +81,13 @@ def _check(spd, value, name, starts):
 @pytest.mark.parametrize("value", [float("nan"), float("inf"), float("-inf")])
 @pytest.mark.parametrize("name", LISTS)
 def test_starts_before_the_sample(spd, value, name):
-    _check(spd, value, name, list(range(-48, 0)))
+    # close to the row end: fewer units follow the sample than make a tile worth
+    # searching whole
+    _check(spd, value, name, list(range(-48, 0)), 2190)
+
+
+@pytest.mark.parametrize("value", [float("nan"), float("inf"), float("-inf")])
+@pytest.mark.parametrize("name", LISTS)
+def test_starts_after_the_sample(spd, value, name):
+    # every unit after the sample's own, in tiles that are searched whole
+    _check(spd, value, name, list(range(16, 64)), 4400)
