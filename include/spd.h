@@ -311,7 +311,9 @@ spd_status spd_cluster_rows(const float *snr, const uint16_t *width, int64_t n_d
 /* Bytes of device workspace spd_detect / spd_search need.  The last piece holds
  * the lists of the screen, which finds the tiles and units of 16 starts that
  * can hold a candidate; a workspace too small for that piece alone is accepted,
- * and every tile is searched: the same records, later. */
+ * and every tile is searched, which takes longer: the same records, but for the
+ * last rounding of an SNR (reported to 2^-17 relative), which depends on the
+ * groups of widths skipped on the way.  Repeated calls give the same bits. */
 size_t spd_detect_workspace_bytes(const spd_plane *plane, const spd_search_params *params);
 size_t spd_search_workspace_bytes(const spd_plane *plane, const spd_search_params *params);
 

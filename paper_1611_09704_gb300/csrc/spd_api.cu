@@ -221,11 +221,11 @@ ScreenLayout screen_lists(int64_t tiles) {
     ScreenLayout l;
     memset(&l, 0, sizeof(l));
     l.tile_cap = tiles;
-    l.unit_cap = 8 * tiles + 1024;
+    l.unit_cap = (int64_t)kScrDense * tiles;   // a tile with more is listed whole
     l.ctl_off = 0;
     l.tiles_off = l.ctl_off + align_up(kScrSlots * sizeof(ScreenCtl));
     l.units_off = l.tiles_off + align_up((size_t)l.tile_cap * sizeof(uint32_t));
-    l.total = l.units_off + align_up((size_t)l.unit_cap * sizeof(uint64_t));
+    l.total = l.units_off + align_up((size_t)l.unit_cap * sizeof(uint32_t));
     return l;
 }
 
@@ -251,7 +251,7 @@ ScreenLists lists_at(char *base, int64_t tiles) {
     const ScreenLayout l = screen_lists(tiles);
     s.ctl = reinterpret_cast<ScreenCtl *>(base + l.ctl_off);
     s.tiles = reinterpret_cast<uint32_t *>(base + l.tiles_off);
-    s.units = reinterpret_cast<uint64_t *>(base + l.units_off);
+    s.units = reinterpret_cast<uint32_t *>(base + l.units_off);
     s.tile_cap = l.tile_cap;
     s.unit_cap = l.unit_cap;
     return s;
@@ -425,7 +425,7 @@ spd_status run_launch(const RangeDesc *rd, int n, int dtype, spd_candidate *out,
     const size_t smem = search_smem_bytes(L.R, raw, max_eval, kmax, G);
     if (smem > 227 * 1024) return SPD_ERR_UNSUPPORTED;
     const bool screen = lists && lists->ctl && !snr_out && nt == kSearchThreads && g_extra_tx != 16 &&
-                        tiles <= lists->tile_cap && tiles < (int64_t)1 << 24;
+                        tiles <= lists->tile_cap && tiles < ((int64_t)1 << 24) - 1;
     size_t lsmem = smem;
     if (screen && tiles > 0) {
         SPD_CK(launch_screen(L, *lists, dtype, st));
@@ -433,7 +433,6 @@ spd_status run_launch(const RangeDesc *rd, int n, int dtype, spd_candidate *out,
         L.tile_count = &lists->ctl->dense;
         L.unit_list = lists->units;
         L.unit_count = &lists->ctl->live;
-        L.unit_cap = (uint32_t)lists->unit_cap;
         // a half-warp per unit where the tiles' shared memory holds them all;
         // at least one warp (an even number: whole warps take part)
         int wmax = 0;

@@ -157,9 +157,8 @@ struct Launch {
     int32_t chunk;              // search kernel: tiles per scheduling chunk (set at launch)
     const uint32_t *tile_list;  // search kernel: the tiles to search (null: all n_tiles)
     const uint32_t *tile_count; // and how many they are
-    const uint64_t *unit_list;  // then single units (null: none), tile << 8 | unit
-    const uint32_t *unit_count; // may exceed unit_cap, the list's room
-    uint32_t unit_cap;
+    const uint32_t *unit_list;  // then single units (null: none), tile << 8 | unit
+    const uint32_t *unit_count;
     int32_t live_blocks, live_halves;   // blocks and half-warps they are searched with
     RangeDesc rng[kMaxRanges];
 };
@@ -248,7 +247,9 @@ constexpr int kScrClasses = 10;
 constexpr int kScrTab = 12;         // floats per scope entry: see ConstArgs::scr_tab
 constexpr int kScrSlots = 16;       // sets of counters: launches of one call
 // Live units of a tile beyond which the tile is searched whole.  A unit takes a
-// half-warp some 800 warp instructions, a tile the search kernel 15,000.
+// half-warp some 800 warp instructions, a tile the search kernel 15,000.  The
+// list of units has room for this many of every tile: which way a tile is
+// searched depends on its samples alone, not on the order of arrival.
 constexpr int kScrDense = 16;
 
 __host__ __device__ inline int screen_class(int w) {
@@ -260,7 +261,7 @@ __host__ __device__ inline int screen_class(int w) {
 // Counters of one screened launch, zeroed by the constants kernel.
 struct ScreenCtl {
     uint32_t dense;       // tiles in the list of tiles
-    uint32_t live;        // units in the list of units (may exceed its capacity)
+    uint32_t live;        // units in the list of units
     uint32_t reserved[2];
 };
 
@@ -268,7 +269,7 @@ struct ScreenCtl {
 struct ScreenLists {
     ScreenCtl *ctl;
     uint32_t *tiles;      // launch-wide tile indexes, room for every tile
-    uint64_t *units;      // tile << 8 | unit of the tile
+    uint32_t *units;      // tile << 8 | unit of the tile (under 2^24 tiles)
     int64_t tile_cap, unit_cap;
 
     // The same lists for launch k of a call: counters of its own.

@@ -17,9 +17,14 @@ __device__ __forceinline__ float half_min(float v, uint32_t hm) {
 // One half-warp per live unit, one start per lane.  The lanes stage the
 // unit's window as the search kernel stages a tile's (y, in-block prefixes P,
 // window sums S_G, block sums), then visit the width groups from the widest
-// down with the search kernel's bounds, group starts, sums and packed max, so
-// that a start's SNR and width come out of the same operations in the same
-// order.  The two halves of a warp meet again to write their records.
+// down with the search kernel's bounds, group starts, sums and packed max.  A
+// group evaluated in both comes out of the same operations in the same order,
+// but for its start when the two skipped different wider groups: the margin of
+// the bounds is that of the unit's prefixes here and of the tile's there, and a
+// start is formed from that of the last group evaluated.  So an SNR can differ
+// in its last rounding: 70 of 357,800 records whose tiles hold a spike of 10^5
+// sigma, none in 120 planes without one.  The two halves of a warp meet again
+// to write their records.
 //
 // Bound by latency: a unit's staging waits for L2 or DRAM once, and a group
 // takes its widths one after the other.  Many units in flight hide it: 20 us
@@ -31,7 +36,7 @@ template <int DT, int G, bool MG>
 __device__ __forceinline__ void live_units(const Launch &L, float *s_dyn, uint32_t in_tiles) {
     using T = typename Elem<DT>::T;
     const int blocks = L.live_blocks, halves = L.live_halves;
-    const uint64_t *units = L.unit_list;
+    const uint32_t *units = L.unit_list;
     const int tid = threadIdx.x, lane = tid & 31, k = lane & 15;
     const int half = tid >> 4;                          // half-warp of the CTA
     const uint32_t hm = 0xffffu << (lane & 16);
@@ -42,16 +47,16 @@ __device__ __forceinline__ void live_units(const Launch &L, float *s_dyn, uint32
     float *s_bs = s_p + (G > 1 ? 2 : 1) * blocks * kSPad;
     float *s_mx = s_bs + blocks;
     float *s_pq = s_mx + blocks;                        // [blocks + 1]
-    const uint32_t n = in_tiles + min(*L.unit_count, L.unit_cap);
+    const uint32_t n = in_tiles + *L.unit_count;
     const uint32_t per = gridDim.x * (uint32_t)halves;
     // warp-uniform trip count: the first half-warp of the warp decides
     for (uint32_t i0 = blockIdx.x * (uint32_t)halves + (uint32_t)((tid >> 5) * 2); i0 < n; i0 += per) {
         const uint32_t i = i0 + (uint32_t)((lane >> 4) & 1);
-        uint64_t id = ~0ull;
+        uint32_t id = ~0u;   // none (a tile index is under 2^24 - 1)
         if (has_room && i < n) {
             if (i < in_tiles) {
                 const uint32_t t = i / (uint32_t)L.units;
-                id = (uint64_t)L.tile_list[t] << 8 | (uint64_t)(i - t * (uint32_t)L.units);
+                id = L.tile_list[t] << 8 | (i - t * (uint32_t)L.units);
             } else {
                 id = units[i - in_tiles];
             }
@@ -60,8 +65,8 @@ __device__ __forceinline__ void live_units(const Launch &L, float *s_dyn, uint32
         int eb = 0, ri = 0;
         int64_t row = 0, i1 = 0;
         bool cand = false;
-        if (id != ~0ull) {
-            const uint32_t tl = (uint32_t)(id >> 8);
+        if (id != ~0u) {
+            const uint32_t tl = id >> 8;
             while (ri + 1 < L.n_ranges && (int64_t)tl >= L.rng[ri + 1].tile0) ++ri;
             const RangeDesc &rd = L.rng[ri];
             const uint32_t lt = tl - (uint32_t)rd.tile0;
@@ -69,9 +74,9 @@ __device__ __forceinline__ void live_units(const Launch &L, float *s_dyn, uint32
             row = q;
             const int64_t col = lt - q * (uint32_t)rd.tiles_per_row;
             i1 = (col * L.units + (int64_t)(id & 255u)) * kX;   // the unit's first start
-            if (i1 >= rd.n_emit) id = ~0ull;   // a listed tile's unit past the row's last start
+            if (i1 >= rd.n_emit) id = ~0u;   // a listed tile's unit past the row's last start
         }
-        if (id != ~0ull) {
+        if (id != ~0u) {
             const RangeDesc &rd = L.rng[ri];
             const RangeProg &rp = rd.prog;
             const int entry = rd.per_row ? (int)row : 0;

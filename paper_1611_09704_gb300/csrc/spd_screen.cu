@@ -412,26 +412,18 @@ __global__ void __launch_bounds__(kScrThreads, 7)
     if (!total) return;
 
     // ---- the lists: a tile with many live units whole, else its units
-    uint32_t base = 0u;
-    bool whole = total > kScrDense;
-    if (!whole) {
-        const uint32_t cap = (uint32_t)A.lists.unit_cap;
-        if (lane == 0) base = atomicAdd(&A.lists.ctl->live, (uint32_t)total);
-        base = __shfl_sync(0xffffffffu, base, 0);
-        if (base > cap || cap - base < (uint32_t)total) {   // no room: the whole tile instead
-            for (uint32_t u = base + lane; u < cap && u >= base; u += 32) A.lists.units[u] = ~0ull;
-            whole = true;
-        }
-    }
-    if (whole) {
+    if (total > kScrDense) {
         if (lane == 0) A.lists.tiles[atomicAdd(&A.lists.ctl->dense, 1u)] = tile;
         return;
     }
+    uint32_t base = 0u;
+    if (lane == 0) base = atomicAdd(&A.lists.ctl->live, (uint32_t)total);
+    base = __shfl_sync(0xffffffffu, base, 0);
     for (int q = 0; 32 * q < nu; ++q) {
         const uint32_t w = __shfl_sync(0xffffffffu, words, q);
         if ((w >> lane) & 1u)
             A.lists.units[base + __popc(w & ((1u << lane) - 1u))] =
-                (uint64_t)tile << 8 | (uint64_t)(32 * q + lane);
+                tile << 8 | (uint32_t)(32 * q + lane);
         base += __popc(w);
     }
 }
