@@ -246,11 +246,22 @@ inline size_t search_smem_bytes(int RM, int raw_bytes, int max_eval, int kmax, i
 constexpr int kScrClasses = 10;
 constexpr int kScrTab = 12;         // floats per scope entry: see ConstArgs::scr_tab
 constexpr int kScrSlots = 16;       // sets of counters: launches of one call
-// Live units of a tile beyond which the tile is searched whole.  A unit takes a
-// half-warp some 800 warp instructions, a tile the search kernel 15,000.  The
-// list of units has room for this many of every tile: which way a tile is
+// Live units of a tile beyond which the tile is searched whole.  A unit stages
+// every block that its widths reach, and the half-warps at work on units are as
+// many as have room for that in shared memory; a tile is staged once for all its
+// units.  So many units took as long as a tile of noise at the search's usual
+// thresholds (512 x 262144 samples, ns per unit and per tile of the launch):
+// widths to 32 0.84 of 24 (28), to 256 by 8 above 16 1.46 of 27 (19), to 512 by
+// 8 3.5 of 40 (11), to 700 6.4 of 43 (7), to 1000 by 16 6.2 of 47 (7), to 2048
+// by 64 13.5 of 38 (3), to 4096 by 16 85 of 98 (1).  With 16 for all of them a
+// search of widths to 4096 at 5.5 sigma took 21.1 ms, 3.2 with every tile whole.
+// The list of units has room for kScrDense of every tile: which way a tile is
 // searched depends on its samples alone, not on the order of arrival.
 constexpr int kScrDense = 16;
+inline int screen_dense(int wmax) {
+    const int d = 330 / (((15 + wmax) >> 4) + 1);
+    return d < 1 ? 1 : d > kScrDense ? kScrDense : d;
+}
 
 __host__ __device__ inline int screen_class(int w) {
     int c = w > 8 ? 1 : 0;

@@ -32,6 +32,7 @@ struct ScreenRange {
     int32_t vec_ok, per_row;
     uint32_t classes;           // bit c: class c holds an evaluated width
     int32_t reach;              // blocks past a unit that its tests read
+    int32_t dense;              // live units up to which a tile is not searched whole
     float threshold;
 };
 
@@ -412,7 +413,7 @@ __global__ void __launch_bounds__(kScrThreads, 7)
     if (!total) return;
 
     // ---- the lists: a tile with many live units whole, else its units
-    if (total > kScrDense) {
+    if (total > rd.dense) {
         if (lane == 0) A.lists.tiles[atomicAdd(&A.lists.ctl->dense, 1u)] = tile;
         return;
     }
@@ -462,6 +463,7 @@ cudaError_t launch_screen(const Launch &L, const ScreenLists &S, int dtype, cuda
         q.per_row = rd.per_row;
         q.tile0 = (uint32_t)rd.tile0;
         q.threshold = rd.threshold;
+        q.dense = screen_dense(rd.prog.wmax);
         q.classes = 0;
         int top = 0;
         for (int g = 0; g < rd.prog.n_groups; ++g) {
