@@ -361,8 +361,8 @@ thread_local uint32_t g_extra_tx = 0;
 // With `lists` (the ranges carrying the screen's tables) the launch is two:
 // the screen, then the search kernel over the tiles it lists and the live
 // units of the rest.  Not with 128-thread tiles (the lists are sized for 256), nor
-// while the test aid makes the copies of every tile run out: then every tile is
-// searched.
+// where no threshold is above 0 (no bound rules anything out then), nor while the
+// test aid makes the copies of every tile run out: then every tile is searched.
 spd_status run_launch(const RangeDesc *rd, int n, int dtype, spd_candidate *out, int64_t cap,
                       spd_result *result, float *snr_out, uint16_t *width_out,
                       int64_t out_stride, int ctas_per_sm, cudaStream_t st, int threads = 0,
@@ -424,8 +424,11 @@ spd_status run_launch(const RangeDesc *rd, int n, int dtype, spd_candidate *out,
     L.units = units;
     const size_t smem = search_smem_bytes(L.R, raw, max_eval, kmax, G);
     if (smem > 227 * 1024) return SPD_ERR_UNSUPPORTED;
-    const bool screen = lists && lists->ctl && !snr_out && nt == kSearchThreads && g_extra_tx != 16 &&
-                        tiles <= lists->tile_cap && tiles < ((int64_t)1 << 24) - 1;
+    bool bounds = false;
+    for (int i = 0; i < n; ++i) bounds = bounds || rd[i].threshold > 0.f;
+    const bool screen = lists && lists->ctl && bounds && !snr_out && nt == kSearchThreads &&
+                        g_extra_tx != 16 && tiles <= lists->tile_cap &&
+                        tiles < ((int64_t)1 << 24) - 1;
     size_t lsmem = smem;
     if (screen && tiles > 0) {
         SPD_CK(launch_screen(L, *lists, dtype, st));

@@ -363,7 +363,8 @@ struct TilePos {
 // False (for the whole CTA) when a bulk copy timed out: it may still land in
 // the shared memory, whose barrier counts it, so neither is to be used again.
 template <int DT, int G, bool MG, int NT, bool PL>
-__device__ __forceinline__ bool search_tiles(const Launch &L, unsigned char *smem) {
+__device__ __forceinline__ bool search_tiles(const Launch &L, unsigned char *smem,
+                                             const uint32_t *list) {
     constexpr int kThreads = NT;
     // units of 16 starts per tile: NT less the halo blocks when the whole
     // window then fits one block per thread (one staging round), else NT
@@ -408,20 +409,19 @@ __device__ __forceinline__ bool search_tiles(const Launch &L, unsigned char *sme
     // where every tile costs the same, takes one fixed run of tiles per CTA
     // instead, without a counter.
     auto counter = [&]() { return reinterpret_cast<unsigned *>(&L.result->reserved0); };
+    // With a list (PL: never) `tile` is an index into it, in chunks of one.
     // the host launches at most n_chunks CTAs (PL: at most n_tiles)
     int64_t tile = PL ? (int64_t)blockIdx.x * L.n_tiles / gridDim.x
-                      : (int64_t)blockIdx.x * L.chunk;
+                      : (int64_t)blockIdx.x * (list ? 1 : L.chunk);
     // the launch's tile count (PL: the end of the CTA's run) and chunk length,
     // read from shared memory where needed (kept out of registers through the
     // search)
     __shared__ long long s_ntiles;
     __shared__ int s_chunk;
-    // with a list (PL: never) `tile` is an index into it, in chunks of one
-    const uint32_t *list = PL ? nullptr : L.tile_list;
     if (tid == 0) {
         s_ntiles = PL ? (int64_t)(blockIdx.x + 1) * L.n_tiles / gridDim.x
                       : list ? (int64_t)*L.tile_count : L.n_tiles;
-        s_chunk = L.chunk;
+        s_chunk = list ? 1 : L.chunk;
     }
     __syncthreads();
     if (list && tile >= s_ntiles) return true;   // more CTAs than listed tiles
@@ -1070,20 +1070,28 @@ __device__ __forceinline__ bool search_tiles(const Launch &L, unsigned char *sme
 // The tiles, then (after a screen) the live units of the tiles not searched
 // whole.  A tile takes its CTA 10 to 20 us however few there are, so when their
 // units make no more than two rounds of the launch's half-warps (some 40 tiles
-// of wmax 256) they are searched as units too.
+// of wmax 256) they are searched as units too.  When 15 of 16 tiles are listed,
+// all are searched, as without a screen: in their order in the plane and in
+// chunks, which spares a listed tile its own claim and, with statistics per row,
+// its own load of constants.  1024 x 524288 samples, every tile full of
+// candidates: 46 widths 7.60 ms by the list and 7.19 so, per row 8.16 and 7.25;
+// widths 1..32 5.71 and 5.20.  With 85 % of the tiles full it is 6.52 and 6.42,
+// per row 7.00 and 6.47, but widths 1..512 (512 x 262144) 6.99 and 7.11.
 template <int DT, int G, bool MG, int NT, bool PL>
 __global__ void __launch_bounds__(NT, 512 / NT) search_kernel(const __grid_constant__ Launch L) {
     extern __shared__ __align__(16) unsigned char smem[];
     uint32_t in_tiles = 0;   // units of listed tiles that the half-warps search
+    const uint32_t *list = nullptr;
     if constexpr (!PL && NT == kSearchThreads) {
         if (L.unit_list) {
-            const uint64_t u = (uint64_t)*L.tile_count * (uint32_t)L.units;
+            const uint64_t n = *L.tile_count, u = n * (uint32_t)L.units;
             if (u <= 2ull * gridDim.x * (uint32_t)L.live_halves) in_tiles = (uint32_t)u;
+            if (in_tiles || 16 * n < 15 * (uint64_t)L.n_tiles) list = L.tile_list;
         }
     }
-    if (!in_tiles && !search_tiles<DT, G, MG, NT, PL>(L, smem)) return;
+    if (!in_tiles && !search_tiles<DT, G, MG, NT, PL>(L, smem, list)) return;
     if constexpr (!PL && NT == kSearchThreads) {
-        if (L.unit_list) {
+        if (list) {
             __syncthreads();
             live_units<DT, G, MG>(L, reinterpret_cast<float *>(smem), in_tiles);
         }
@@ -1110,7 +1118,7 @@ cudaError_t launch_sgn(const Launch &L, bool mg, size_t smem, int ctas_per_sm, c
     const int64_t gmax = (int64_t)sms * per_sm;
     int64_t ch = 16;
     while (ch > 1 && L.n_tiles < 8 * gmax * ch) ch >>= 1;
-    if (PL || L.tile_list) ch = 1;
+    if (PL) ch = 1;
     Launch Lc = L;
     Lc.chunk = (int32_t)ch;
     const int64_t n_chunks = (L.n_tiles + ch - 1) / ch;
