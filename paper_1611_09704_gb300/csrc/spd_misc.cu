@@ -138,21 +138,28 @@ __global__ void boxcar_sums_kernel(const spd_plane p, int w, float *out, int64_t
 // candidates are a ballot mask, the lanes that start a cluster (more than
 // `gap` past the last candidate before them: the previous set bit, else the
 // open cluster's last) form a second mask, and each segment between starts is
-// absorbed with a popcount, its highest set bit, and one warp max (redux)
-// over order-preserving keys of its SNRs.  Every lane holds the same cluster
-// state, so lane 0 alone writes records, and reads the peak's width then: the
-// width plane is not streamed.
+// absorbed with a popcount and its highest set bit.  Every lane holds the same
+// cluster state but for the peak, of which it keeps its own over order-
+// preserving keys; one warp max when the cluster ends finds the lane that writes
+// the record and reads the peak's width: the width plane is not streamed.
 //
-// Bound by the SNR plane's one read.  1024 x 262144 samples: a warp per row
-// left 7 warps per SM and streamed the widths too, 815 us; now 169 us, 6.3
-// TB/s.
+// Bound by the SNR plane's one read where candidates are few.  1024 x 262144
+// samples: a warp per row left 7 warps per SM and streamed the widths too, 815
+// us; now 169 us, 6.3 TB/s.  A cluster that runs through a row is one warp's
+// walk, while the other segments' warps pass over their parts of it.  With a
+// warp max for every step, and no way to take a load at once, such rows took
+// longer than with a warp per row: gap 32, every sample a candidate 3.54 ms (a
+// warp per row 1.95), now 1.85; gap 8 3.56 (1.95) and 2.28.
 constexpr int kClusterWarps = 8;    // segments per CTA
 constexpr int kClusterSteps = 16;   // 32-sample steps loaded at once per warp
 
+// The open cluster: the same in every lane, but for the peak, of which a lane
+// holds the highest of the members it has seen (the earliest among equals).
 struct ClusterState {
-    int first, last, peak_t, members;
+    int first, last, members;
+    unsigned key;
     float peak;
-    unsigned peak_key;
+    int peak_t;
 };
 
 // Monotone map of a non-NaN float to an unsigned key (larger float, larger
@@ -164,10 +171,14 @@ __device__ __forceinline__ unsigned order_key(float f) {
     return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
+// The whole warp: the peak over its lanes; the lane that saw it writes the record.
 __device__ __forceinline__ void emit_cluster(const ClusterState &c, int64_t row,
                                              const uint16_t *wp, spd_cluster *out,
-                                             int64_t capacity, spd_result *result, int lane) {
-    if (lane != 0) return;
+                                             int64_t capacity, spd_result *result) {
+    const unsigned top = __reduce_max_sync(0xffffffffu, c.key);
+    const unsigned at = __reduce_min_sync(0xffffffffu, c.key == top ? (unsigned)c.peak_t : ~0u);
+    if (c.key != top || (unsigned)c.peak_t != at) return;
+    const int w = wp[c.peak_t];   // beside the atomic, not after it
     const unsigned long long idx =
         atomicAdd(reinterpret_cast<unsigned long long *>(&result->count), 1ull);
     if (idx < (unsigned long long)capacity) {
@@ -177,28 +188,62 @@ __device__ __forceinline__ void emit_cluster(const ClusterState &c, int64_t row,
         r.last = c.last;
         r.peak_sample = c.peak_t;
         r.peak_snr = c.peak;
-        r.peak_width = wp[c.peak_t];
+        r.peak_width = w;
         r.members = c.members;
         r.reserved0 = 0;
         out[idx] = r;
     }
 }
 
-// The members M (a lane mask of this step, starting at sample t0) join the
-// open cluster: count, last sample, and the peak (strict: an earlier equal
-// peak stays; within M the lowest lane of the maximum).
+// The members M (a lane mask of this step, starting at sample t0) join the open
+// cluster: count, last sample, and each lane's own peak (key: 0 where the lane's
+// sample is no candidate).
 __device__ __forceinline__ void absorb(ClusterState &c, unsigned M, int t0, unsigned key, float v,
                                        int lane) {
     c.members += __popc(M);
     c.last = t0 + (31 - __clz(M));
     const unsigned mine = ((M >> lane) & 1u) ? key : 0u;
-    const unsigned kmax = __reduce_max_sync(0xffffffffu, mine);
-    if (kmax > c.peak_key) {
-        const int pl = __ffs(__ballot_sync(0xffffffffu, mine == kmax)) - 1;
-        c.peak_key = kmax;
-        c.peak = __shfl_sync(0xffffffffu, v, pl);
-        c.peak_t = t0 + pl;
+    const bool up = mine > c.key;
+    c.key = up ? mine : c.key;
+    c.peak = up ? v : c.peak;
+    c.peak_t = up ? t0 + lane : c.peak_t;
+}
+
+// All the candidates of a load's steps (samples from t0 on) join the open cluster
+// when none of them starts one; else nothing changes and the result is false.
+// One vote for all steps, where the walk below has one or two a step.
+__device__ __forceinline__ bool join_steps(ClusterState &c, bool foreign,
+                                           const float (&v)[kClusterSteps], float thr, int t0,
+                                           int gap, int lane) {
+    int last = c.last, members = 0;
+    bool far = false;
+#pragma unroll
+    for (int k = 0; k < kClusterSteps; ++k) {
+        const unsigned m = __ballot_sync(0xffffffffu, v[k] >= thr);
+        if (m) {
+            far |= t0 + 32 * k + __ffs(m) - 1 - last > gap;
+            if (gap < 31) {   // more than gap samples between two of the step
+                const unsigned below = m & ((1u << lane) - 1u);
+                far |= ((m >> lane) & 1u) && below && lane - (31 - __clz(below)) > gap;
+            }
+            last = t0 + 32 * k + (31 - __clz(m));
+            members += __popc(m);
+        }
     }
+    if (__any_sync(0xffffffffu, far)) return false;
+    c.last = last;
+    if (foreign) return true;
+    c.members += members;
+#pragma unroll
+    for (int k = 0; k < kClusterSteps; ++k) {
+        const unsigned key = v[k] >= thr ? order_key(v[k]) : 0u;
+        if (key > c.key) {
+            c.key = key;
+            c.peak = v[k];
+            c.peak_t = t0 + 32 * k + lane;
+        }
+    }
+    return true;
 }
 
 __global__ void __launch_bounds__(32 * kClusterWarps) cluster_kernel(
@@ -213,7 +258,8 @@ __global__ void __launch_bounds__(32 * kClusterWarps) cluster_kernel(
     const float *sp = snr + row * stride;
     const uint16_t *wp = width + row * stride;
     bool open = false, foreign = false, looked = a == 0;
-    ClusterState c{0, 0, 0, 0, 0.f, 0u};
+    int quiet = 0;   // loads since one in which a cluster started
+    ClusterState c{0, 0, 0, 0u, 0.f, 0};
     // the segment, then on past its end while an own cluster is open
     for (int64_t base = a; base < n; base += 32 * kClusterSteps) {
         if (base >= b && (!open || foreign || base - c.last > gap)) break;
@@ -222,14 +268,19 @@ __global__ void __launch_bounds__(32 * kClusterWarps) cluster_kernel(
 #pragma unroll
         for (int k = 0; k < kClusterSteps; ++k) {
             const int64_t t = base + 32 * k + lane;
-            v[k] = t < n ? __ldcs(sp + t) : -INFINITY;
+            v[k] = t < n ? __ldcs(sp + t) : __int_as_float(0x7fc00000);   // NaN: not a candidate
         }
 #pragma unroll
-        for (int k = 0; k < kClusterSteps; ++k) any |= v[k] >= thr;   // NaN: not a candidate
+        for (int k = 0; k < kClusterSteps; ++k) any |= v[k] >= thr;
         if (!__any_sync(0xffffffffu, any)) continue;
+        // worth trying after some loads without a start: a load that has one is
+        // gone over twice (gap 8, clusters of 500 samples: 1.13 ms never tried,
+        // 1.20 after four such loads, 1.48 after two)
+        if (quiet >= 4 && join_steps(c, foreign, v, thr, (int)base, gap, lane)) continue;
+        ++quiet;
 #pragma unroll
         for (int k = 0; k < kClusterSteps; ++k) {
-            const bool cand = v[k] >= thr && base + 32 * k + lane < n;
+            const bool cand = v[k] >= thr;
             const unsigned m = __ballot_sync(0xffffffffu, cand);
             if (!m) continue;
             const int t0 = (int)(base + 32 * k);
@@ -246,34 +297,40 @@ __global__ void __launch_bounds__(32 * kClusterWarps) cluster_kernel(
                     c.last = t1 - 1;   // any sample at most gap before it
                 }
             }
+            const unsigned key = cand ? order_key(v[k]) : 0u;
+            // a gap of 31 or more spans what lies between two set bits: all join
+            if (gap >= 31 && open && t0 + __ffs(m) - 1 - c.last <= gap) {
+                absorb(c, m, t0, key, v[k], lane);
+                continue;
+            }
             // does this lane's candidate start a cluster?
             const unsigned below = m & ((1u << lane) - 1u);
             const bool has_prev = below != 0u || open;
             const int prev = below ? t0 + (31 - __clz(below)) : c.last;
             const bool start = cand && (!has_prev || (t0 + lane) - prev > gap);
             unsigned S = __ballot_sync(0xffffffffu, start);
-            const unsigned key = cand ? order_key(v[k]) : 0u;
             // members before the first start continue the open cluster
             const int fs = S ? __ffs(S) - 1 : 32;
             const unsigned cont = fs == 32 ? m : (m & ((1u << fs) - 1u));
-            if (cont) absorb(c, cont, t0, key, v[k], lane);
+            if (cont) absorb(c, cont, t0, key, v[k], lane);   // a foreign one's is never written
+            if (S) quiet = 0;
             while (S) {
                 const int s0 = __ffs(S) - 1;
                 S &= S - 1u;
                 const int e = S ? __ffs(S) - 1 : 32;
                 const unsigned seg = m & (0xffffffffu << s0) & (e == 32 ? 0xffffffffu : ((1u << e) - 1u));
-                if (open && !foreign) emit_cluster(c, row, wp, out, capacity, result, lane);
+                if (open && !foreign) emit_cluster(c, row, wp, out, capacity, result);
                 open = t0 + s0 < b;   // one that starts past the segment is the next one's
                 foreign = false;
                 if (!open) return;
                 c.first = t0 + s0;
                 c.members = 0;
-                c.peak_key = 0u;
+                c.key = 0u;
                 absorb(c, seg, t0, key, v[k], lane);
             }
         }
     }
-    if (open && !foreign) emit_cluster(c, row, wp, out, capacity, result, lane);
+    if (open && !foreign) emit_cluster(c, row, wp, out, capacity, result);
 }
 
 }  // namespace
