@@ -327,6 +327,7 @@ __global__ void __launch_bounds__(kDdThreads, 2) dedisperse_kernel(
             w += 4u * tid;
 #pragma unroll
             for (int q = 0; q < DMS / 4; ++q) {
+                if (4 * q >= nd) break;  // past the block's last trial
                 const int4 d4 = dv[q];   // four trials' offsets, one broadcast load
                 const int o[4] = {d4.x, d4.y, d4.z, d4.w};
 #pragma unroll
@@ -355,6 +356,7 @@ __global__ void __launch_bounds__(kDdThreads, 2) dedisperse_kernel(
             const int4 *dv = reinterpret_cast<const int4 *>(s_dl[c]);
 #pragma unroll
             for (int q = 0; q < DMS / 4; ++q) {
+                if (4 * q >= nd) break;
                 const int4 d4 = dv[q];   // trials past the block's last read offset 0
                 const int o[4] = {d4.x, d4.y, d4.z, d4.w};
                 T v[4][PER];
