@@ -435,20 +435,24 @@ cudaError_t launch_dd(const spd_plane *fb, const int32_t *delays, int64_t n_dm, 
     return cudaGetLastError();
 }
 
-// 4 outputs of 16 trials per thread where that gives two CTAs per SM or more
-// (both fit), 2 outputs where that gives 64; else CTAs of an eighth of that,
-// so that a small plane still fills the chip: 512 channels x 16 trials x 8192
-// outputs (16 of the middle shape) 2.73 -> 0.59 ms, but 100 x 64 x 30000 (236
-// of them) 0.12 ms in the middle shape and 0.18 in the small one, which forms
-// each window for 4 trials only.
+// The middle shape, 2 outputs of 16 trials per thread, where its CTAs all fit the
+// chip at once (two per SM) but are not few.  Beyond that 4 outputs: 256 channels
+// FP32, 48 trials x 60000 (354 CTAs of the middle shape) 277 us in the middle
+// shape, 228 in the large one; 100 x 30000 (413) 270 and 216; but 256 x 8192
+// (256) 143 and 164, 48 x 30000 (177) 160 and 186.  With few, CTAs of an eighth
+// of the middle shape, which form each window for 4 trials only: FP32 48 x 16384
+// (96) 135 in the middle shape, 165 in the small one, 256 x 2000 (64) 119 and
+// 113, 100 x 4000 (56) 125 and 96, 16 x 30000 (59) 178 and 112; FP16 124 and 142
+// at 64, 130 and 127 at 56.
 template <int DT>
 cudaError_t launch_dd_dt(const spd_plane *fb, const int32_t *delays, int64_t n_dm, void *out,
                          int out_dt, int64_t n_out, int64_t out_stride, spd_result *status,
                          cudaStream_t s) {
     const int64_t b16 = (n_dm + 15) / 16;
-    if ((n_out + 1023) / 1024 * b16 >= 304)
+    const int64_t ctas = (n_out + 511) / 512 * b16;
+    if (ctas > 304)
         return launch_dd<DT, 4, 16>(fb, delays, n_dm, out, out_dt, n_out, out_stride, status, s);
-    if ((n_out + 511) / 512 * b16 >= 64)
+    if (ctas >= 64)
         return launch_dd<DT, 2, 16>(fb, delays, n_dm, out, out_dt, n_out, out_stride, status, s);
     return launch_dd<DT, 1, 4>(fb, delays, n_dm, out, out_dt, n_out, out_stride, status, s);
 }
