@@ -4,8 +4,9 @@ For a given batch (the DM ranges' shapes, storage type, width sets,
 thresholds and sigma modes) every candidate launch shape -- persistent CTAs
 per SM, width-group size (widths per pass between bounds) and tile length
 (threads per CTA: a tile is 16 starts per thread less the halo's blocks) --
-is timed on the device with CUDA events, and the fastest is kept.  Results are cached in a JSON file keyed by the device
-and a hash of the batch description, so a serving process tunes once.
+is timed on the device with CUDA events, and the fastest is kept.  Results are
+cached in a JSON file keyed by a hash of the device, the batch description and the
+launch rules' version, so a serving process tunes once.
 """
 from __future__ import annotations
 
@@ -18,15 +19,22 @@ CANDIDATES = [{"ctas_per_sm": c, "group_scale": g, "tile_threads": t}
               for t in (256, 128) for c in (0, 1) for g in (1, 2, 4)]
 
 
+# What the timings of a cache entry depend on beyond the batch: raised when the
+# launches change so much that an older choice may be a bad one.  2: a screen
+# before the search, which 128-thread tiles go without (four ranges, 1.6e9 samples
+# of noise: 33 ms a launch against 1.4 with the screen).
+RULES = 2
+
+
 def batch_key(specs, device_name: str) -> str:
-    """Stable key of a batch: device, storage type, shapes and search parameters."""
+    """Stable key of a batch: device, storage type, shapes, search parameters, rules."""
     desc = []
     for r in specs:
         x = r.x.data if hasattr(r.x, "n_samp") else r.x
         n_samp = r.x.n_samp if hasattr(r.x, "n_samp") else x.shape[1]
         desc.append([str(x.dtype), int(x.shape[0]), int(n_samp), [int(w) for w in r.widths],
                      float(r.threshold), int(r.sigma_mode), int(r.scope), int(r.nmax)])
-    blob = json.dumps([device_name, desc], sort_keys=True).encode()
+    blob = json.dumps([device_name, desc, RULES], sort_keys=True).encode()
     return hashlib.sha1(blob).hexdigest()
 
 
