@@ -204,8 +204,8 @@ DetLayout det_layout(int64_t entries, int n_eval) {
 // one piece after everything else a call keeps in its workspace.  A caller
 // whose workspace holds all but this piece gets the search without a screen.
 struct ScreenLayout {
-    size_t tab_off, grp_off, ctl_off, tiles_off, units_off, total;
-    int64_t tile_cap, unit_cap;
+    size_t ctl_off, tiles_off, units_off, total;
+    int64_t tile_cap;
 };
 
 // Most tiles of the search kernel (256 threads: at least 192 units of 16
@@ -221,11 +221,11 @@ ScreenLayout screen_lists(int64_t tiles) {
     ScreenLayout l;
     memset(&l, 0, sizeof(l));
     l.tile_cap = tiles;
-    l.unit_cap = (int64_t)kScrDense * tiles;   // a tile with more is listed whole
     l.ctl_off = 0;
     l.tiles_off = l.ctl_off + align_up(kScrSlots * sizeof(ScreenCtl));
     l.units_off = l.tiles_off + align_up((size_t)l.tile_cap * sizeof(uint32_t));
-    l.total = l.units_off + align_up((size_t)l.unit_cap * sizeof(uint32_t));
+    // a tile with more units is listed whole
+    l.total = l.units_off + align_up((size_t)(kScrDense * tiles) * sizeof(uint32_t));
     return l;
 }
 
@@ -253,7 +253,6 @@ ScreenLists lists_at(char *base, int64_t tiles) {
     s.tiles = reinterpret_cast<uint32_t *>(base + l.tiles_off);
     s.units = reinterpret_cast<uint32_t *>(base + l.units_off);
     s.tile_cap = l.tile_cap;
-    s.unit_cap = l.unit_cap;
     return s;
 }
 

@@ -1,7 +1,6 @@
 // spd_device.cuh -- device helpers shared by the detect kernels: packed
 // (SNR, code) floats, packed f32x2 arithmetic, 1-D bulk (TMA) copies with a
-// time-bounded mbarrier wait, vector loads of stored samples and
-// double-float sums.
+// time-bounded mbarrier wait, and vector loads of stored samples.
 #pragma once
 #include "spd_internal.cuh"
 
@@ -171,20 +170,6 @@ __device__ __forceinline__ void load_centred(float *v, const typename Elem<DT>::
             v[e] = q < have ? x : -INFINITY;
         }
     }
-}
-
-// ------------------------------------------------------- double-float sums
-
-__device__ __forceinline__ float2 two_sum(float a, float b) {
-    const float s = __fadd_rn(a, b);
-    const float bb = __fsub_rn(s, a);
-    const float e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-    return make_float2(s, e);
-}
-__device__ __forceinline__ float2 df_add(float2 a, float2 b) {
-    float2 s = two_sum(a.x, b.x);
-    const float lo = __fadd_rn(s.y, __fadd_rn(a.y, b.y));
-    return two_sum(s.x, lo);
 }
 
 }  // namespace

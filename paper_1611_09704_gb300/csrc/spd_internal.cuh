@@ -59,7 +59,7 @@ inline unsigned *merge_counter(MsdPart *scratch, int n_scratch) {
     return reinterpret_cast<unsigned *>(scratch + n_scratch - 1);
 }
 
-// Arguments of the sigma_Nmax pass (Eq. 5): tiles of 4096 starts per row.
+// Arguments of the sigma_Nmax pass (Eq. 5): tiles of 8192 starts per row.
 struct NmaxArgs {
     const void *data;
     int64_t n_dm, n_samp, stride;
@@ -69,7 +69,7 @@ struct NmaxArgs {
     int vec_ok;                 // rows aligned for 4-element vector loads
     int nmax;
     int nb;                     // staged blocks of 16 samples per tile
-    int64_t tiles_per_row;      // partials per row (each covers up to 8 tiles of 4096 starts)
+    int64_t tiles_per_row;      // partials per row (each covers up to 4 tiles of 8192 starts)
     MsdPart *parts;             // [n_dm * tiles_per_row]
 };
 
@@ -281,7 +281,7 @@ struct ScreenLists {
     ScreenCtl *ctl;
     uint32_t *tiles;      // launch-wide tile indexes, room for every tile
     uint32_t *units;      // tile << 8 | unit of the tile (under 2^24 tiles)
-    int64_t tile_cap, unit_cap;
+    int64_t tile_cap;
 
     // The same lists for launch k of a call: counters of its own.
     ScreenLists slot(int k) const {

@@ -114,22 +114,6 @@ struct Acc2 {
         }
     }
 
-    // (T, S) of v[0..7] per lane by their definition: the sum, then the
-    // squared deviations from the group mean.  Returns U = -T and S8.
-    static __device__ __forceinline__ void direct_8(const float2 *v, float2 &U, float2 &S8) {
-        const float2 t = __fadd2_rn(__fadd2_rn(__fadd2_rn(v[0], v[1]), __fadd2_rn(v[2], v[3])),
-                                    __fadd2_rn(__fadd2_rn(v[4], v[5]), __fadd2_rn(v[6], v[7])));
-        const float2 nm = __fmul2_rn(t, f2(-0.125f));   // minus the mean
-        float2 d = __fadd2_rn(v[0], nm);
-        S8 = __fmul2_rn(d, d);
-#pragma unroll
-        for (int k = 1; k < 8; ++k) {
-            d = __fadd2_rn(v[k], nm);
-            S8 = __ffma2_rn(d, d, S8);
-        }
-        U = __fmul2_rn(t, f2(-1.f));
-    }
-
     // Eq. 2: fold a set of 8 per lane (sum -U, S8) into the running sets.
     __device__ __forceinline__ void fold8(float2 U, float2 S8) {
         const float2 m1 = f2(-1.f);
@@ -569,10 +553,11 @@ __global__ void __launch_bounds__(256) consts_kernel(const ConstArgs a,
 // one scope entry when asked for (consts.msd not null).  `arrived` is 0 at
 // launch and again after it.  With `state` the parts join a running MSD.
 //
-// Bound by the latency of its FP64 divisions: 25 us for 32768 parts (4096 x
-// 524288), what the three launches it replaced took without the gaps between
-// them; the searches of 64 x 65536 samples, bound by the host, gain the three
-// launches (a fold, a memset and the constants) it and the partials save.
+// Bound by the latency of its chain: the parts from L2, a dozen FP64 instructions
+// a thread (block_merge), the scratch, and the constants: 12 us for 32768 parts
+// (4096 x 524288).  With the paper's two divisions per fold it was 25, what the
+// three launches it replaced took without the gaps between them.  It and the
+// partials save a search three launches (a fold, a memset and the constants).
 __global__ void __launch_bounds__(kMsdThreads)
     msd_merge_kernel(const MsdPart *parts, int64_t n_parts, int64_t per, MsdPart *scratch,
                      unsigned *arrived, int nmax, MsdPart *state, spd_msd_stats *out,

@@ -398,9 +398,13 @@ __global__ void __launch_bounds__(kScrThreads, 7)
         };
         keep(rr);
         if (rr < mirror) keep(rr + ring);
-        // the prefixes are off by some 30 roundings of the tile's largest
-        // partial sum so far at most (in-block 16, the scan, the running
-        // total, and their uses): the margin is six times that
+        // margin for the rounding of the prefixes: 200 unit roundoffs of the
+        // tile's largest partial sum so far.  The same additions restated on the
+        // host beside FP64 put a difference of two prefixes off by 9 at most on
+        // noise, offsets of 0.6 and 100 sigma, drifts and spikes of 10^4 and 10^5
+        // sigma.  It is no bound of the worst case: a constant with spikes of
+        // +-10^5 in every block, whose additions all round the same way, is off
+        // by 940 (and the SNRs' own sums with it)
         const float big = fmaxf(fabsf(mx), fabsf(mn));
         const uint32_t top = __reduce_max_sync(0xffffffffu, big < kInf ? __float_as_uint(big) : 0u);
         mag = fmaxf(mag, __uint_as_float(top));

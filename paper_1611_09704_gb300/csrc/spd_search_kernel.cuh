@@ -829,8 +829,8 @@ __device__ __forceinline__ bool search_tiles(const Launch &L, unsigned char *sme
         // ---- search of the unit's 16 starts (widest group first)
         const float thr = rd.threshold;
         const float minC = PL ? 0.f : s_mn[tid];
-        // the FP32 prefix values are off by at most ~30 roundings of the
-        // tile's largest partial sum: the prefix bound adds twice that
+        // margin for the rounding of the FP32 prefixes: 130 unit roundoffs of the
+        // tile's largest partial sum, as in the screen
         const float cslack = fmaf(8e-6f, __int_as_float(s_mag), 1e-30f) - minC;
         const float pq0 = PL ? 0.f : s_pq[tid];
         const float *yb = s_y + kSPad * tid;
