@@ -6,6 +6,8 @@
 // coupling Sec. 3 names as future work).
 #include "spd_internal.cuh"
 
+#include <type_traits>
+
 namespace spd {
 void note_cuda_error(int e);
 }
@@ -327,7 +329,6 @@ __global__ void __launch_bounds__(kDdThreads, 2) dedisperse_kernel(
             w += 4u * tid;
 #pragma unroll
             for (int q = 0; q < DMS / 4; ++q) {
-                if (4 * q >= nd) break;  // past the block's last trial
                 const int4 d4 = dv[q];   // four trials' offsets, one broadcast load
                 const int o[4] = {d4.x, d4.y, d4.z, d4.w};
 #pragma unroll
@@ -346,17 +347,16 @@ __global__ void __launch_bounds__(kDdThreads, 2) dedisperse_kernel(
                 }
             }
         };
-        // a wide spread: channel c straight from global memory, the loads of
-        // four trials in flight at a time
-        auto add_global = [&](int c) {
+        // a wide spread: channel c straight from global memory, for the first
+        // 4 QUADS trials; the loads of all in flight together
+        auto add_global_to = [&](auto quads, int c) {
             const T *row = fb + (c0 + c) * fb_stride + s_lo[c] + t0 + tid;
             const float sc = has_sc ? __ldg(scale + c0 + c) : 1.f;
             const float of = (has_sc && offset) ? __ldg(offset + c0 + c) : 0.f;
             const int left = (int)min(n_out - t0 - tid, (int64_t)kSpan);   // outputs from the first
             const int4 *dv = reinterpret_cast<const int4 *>(s_dl[c]);
 #pragma unroll
-            for (int q = 0; q < DMS / 4; ++q) {
-                if (4 * q >= nd) break;
+            for (int q = 0; q < decltype(quads)::value; ++q) {
                 const int4 d4 = dv[q];   // trials past the block's last read offset 0
                 const int o[4] = {d4.x, d4.y, d4.z, d4.w};
                 T v[4][PER];
@@ -373,6 +373,16 @@ __global__ void __launch_bounds__(kDdThreads, 2) dedisperse_kernel(
                         a = __fadd_rn(a, fb_value<DT>(&v[e][j], has_sc, sc, of));
                     }
             }
+        };
+        // a block of few trials reads no others: 128 x 3 x 262144 FP32 with delays
+        // to 1000 pc/cm3 280 us in the middle shape reading 16, 173 so.  (A test
+        // before every four trials keeps their loads from overlapping: 1024 x 16 x
+        // 65536 at the same delays 1.04 ms without, 2.01 with it; in `add`, 216 x
+        // 28 x 48704 172 and 229 us.  The middle shape has no registers to spare.)
+        auto add_global = [&](int c) {
+            if (PER == 4 && nd <= 4) add_global_to(std::integral_constant<int, 1>{}, c);
+            else if (PER == 4 && nd <= 8) add_global_to(std::integral_constant<int, DMS < 8 ? 1 : 2>{}, c);
+            else add_global_to(std::integral_constant<int, DMS / 4>{}, c);
         };
         const uint32_t w0 = (uint32_t)__cvta_generic_to_shared(s_w);
         const uint32_t x0 = (uint32_t)__cvta_generic_to_shared(s_x);
