@@ -95,9 +95,11 @@ __device__ __forceinline__ void cp_async_wait_all() {
 // and whole blocks of the sums formed without bound checks (2.8 per add).  200
 // x 117 x 60001 FP16: 583 -> 300 us (16-bit windows staged as they are).
 // Trials too far apart to share a window, 200 x 32 x 16000: 0.51 -> 0.14 ms
-// (the loads of four trials in flight).
+// (the loads of four trials in flight).  The small shape fits four CTAs per SM in
+// shared memory, and is held to the registers for that: 512 x 16 x 30000 FP32 (472
+// CTAs) 363 us with three of 68 registers, 230 so.
 template <int DT, int PER, int DMS>
-__global__ void __launch_bounds__(kDdThreads, 2) dedisperse_kernel(
+__global__ void __launch_bounds__(kDdThreads, PER == 1 ? 4 : 2) dedisperse_kernel(
     const typename Elem<DT>::T *fb, int64_t n_chan, int64_t n_samp, int64_t fb_stride,
     const float *scale, const float *offset, const int32_t *delays, int64_t n_dm, void *out,
     int out_dt, int64_t n_out, int64_t out_stride, spd_result *status) {
