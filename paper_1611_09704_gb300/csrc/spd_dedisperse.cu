@@ -449,13 +449,13 @@ cudaError_t launch_dd(const spd_plane *fb, const int32_t *delays, int64_t n_dm, 
 
 // The middle shape, 2 outputs of 16 trials per thread, where its CTAs all fit the
 // chip at once (two per SM) but are not few.  Beyond that 4 outputs: 256 channels
-// FP32, 48 trials x 60000 (354 CTAs of the middle shape) 277 us in the middle
-// shape, 228 in the large one; 100 x 30000 (413) 270 and 216; but 256 x 8192
-// (256) 143 and 164, 48 x 30000 (177) 160 and 186.  With few, CTAs of an eighth
+// FP32, 48 trials x 60000 (354 CTAs of the middle shape) 260 us in the middle
+// shape, 227 in the large one; 100 x 30000 (413) 263 and 212; but 256 x 8192
+// (256) 140 and 154, 48 x 30000 (177) 157 and 177.  With few, CTAs of an eighth
 // of the middle shape, which form each window for 4 trials only: FP32 48 x 16384
-// (96) 135 in the middle shape, 165 in the small one, 256 x 2000 (64) 119 and
-// 113, 100 x 4000 (56) 125 and 96, 16 x 30000 (59) 178 and 112; FP16 124 and 142
-// at 64, 130 and 127 at 56.
+// (96) 126 in the middle shape and 170 in the small one, 256 x 2000 (64) 112 and
+// 118, 100 x 4000 (56) 117 and 99, 16 x 30000 (59) 140 and 118; FP16 113 and 144 at
+// 64, 122 and 126 at 56.
 template <int DT>
 cudaError_t launch_dd_dt(const spd_plane *fb, const int32_t *delays, int64_t n_dm, void *out,
                          int out_dt, int64_t n_out, int64_t out_stride, spd_result *status,
