@@ -183,6 +183,11 @@ __global__ void __launch_bounds__(kScrThreads, 7)
     const int entry = rd.per_row ? (int)row : 0;
     const int64_t emit = min(rd.n_emit - t0, (int64_t)A.units * kX);
     if (emit <= 0 || rd.flags[entry]) return;
+    // the tile's limit of live units, not held in a register through the walk (2048
+    // x 524288 FP16 with a scale, 46 widths: 619 us with a constant limit, 627 with
+    // the launch's read at the end); widths to 256 all have the same
+    __shared__ int s_dense[kScrWarps];
+    if (kTop > 5 && lane == 0) s_dense[warp] = rd.dense;
     const int nu = (int)((emit + kX - 1) / kX);
     const int reach = rd.reach;
     const int nb = nu + reach;
@@ -295,11 +300,10 @@ __global__ void __launch_bounds__(kScrThreads, 7)
             }
         }
         // a prefix that is not finite (a sample before the unit that is not)
-        // rules nothing out, nor does an energy: a maximum of two would drop a
-        // NaN, so each is tested
+        // rules nothing out, nor does an energy
         bool live = all | !(fabsf(base) < kInf) | !(m + base < 0.f);
-        live |= !(ha < h0) | !(hb < h0);
-        live |= !(fmaxf(x0, x1) - g1 + base < 0.f) & (!(ha + eb.x < h1) | !(ea.y + hc < h1));
+        live |= !(fmax_nan(ha, hb) < h0);
+        live |= !(fmaxf(x0, x1) - g1 + base < 0.f) & !(fmax_nan(ha + eb.x, ea.y + hc) < h1);
         live &= 32 * rt + lane < nu;
         const uint32_t bal = __ballot_sync(0xffffffffu, live);
         if (lane == rt) words = bal;
@@ -417,7 +421,7 @@ __global__ void __launch_bounds__(kScrThreads, 7)
     if (!total) return;
 
     // ---- the lists: a tile with many live units whole, else its units
-    if (total > rd.dense) {
+    if (total > (kTop > 5 ? s_dense[warp] : kScrDense)) {
         if (lane == 0) A.lists.tiles[atomicAdd(&A.lists.ctl->dense, 1u)] = tile;
         return;
     }
