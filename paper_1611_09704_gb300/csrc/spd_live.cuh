@@ -182,7 +182,8 @@ __device__ __forceinline__ void live_units(const Launch &L, float *s_dyn, uint32
                 // energy of the blocks the windows lie in: this group's and all narrower ones'
                 if (s_pq[1 + ((14 + end) >> 4)] * 1.000008f * gt.y < lim2) break;
                 float rmax = -INFINITY;
-                for (int b = (g.off + d) >> 4; b <= (15 + end) >> 4; ++b) rmax = fmaxf(rmax, s_mx[b]);
+                for (int b = (g.off + d) >> 4; b <= (15 + end) >> 4; ++b)
+                    rmax = fmax_nan(rmax, s_mx[b]);
                 if (fmax_nan(rmax + cslack, 0.f) * gt.x < lim_lo) continue;   // NaN never prunes
                 if (MG && (g.widx0 >> 6) != cur) {
                     if (cur >= 0 && trunc17(cb) >= trunc17(ob)) {

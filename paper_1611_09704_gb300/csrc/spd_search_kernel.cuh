@@ -805,7 +805,7 @@ __device__ __forceinline__ bool search_tiles(const Launch &L, unsigned char *sme
                             if (j >= (1 << kl)) break;
                             const int b = min(c + j, R - 1);
                             const float Pb = ((b >> 5) == chunk ? (chunk ? pre : 0.f) : pre_n) + s_ex[b];
-                            m = fmaxf(m, Pb + s_rh[b]);
+                            m = fmax_nan(m, Pb + s_rh[b]);
                             if (j == 1) s_mx[RM + c] = m;
                             if (j == 3) s_mx[2 * RM + c] = m;
                             if (j == 7) s_mx[3 * RM + c] = m;
@@ -821,7 +821,7 @@ __device__ __forceinline__ bool search_tiles(const Launch &L, unsigned char *sme
                 const float *lo = s_mx + (lv - 1) * RM;
                 const int h = 1 << (lv - 1);
                 for (int c = tid; c < R; c += kThreads)
-                    s_mx[lv * RM + c] = fmaxf(lo[c], lo[min(c + h, R - 1)]);
+                    s_mx[lv * RM + c] = fmax_nan(lo[c], lo[min(c + h, R - 1)]);
                 __syncthreads();
             }
         }
@@ -873,10 +873,10 @@ __device__ __forceinline__ bool search_tiles(const Launch &L, unsigned char *sme
             if (!PL) {
                 float rmax;
                 if (gb.y >= 0) {
-                    rmax = fmaxf(s_mx[tid + ga.z], s_mx[tid + ga.w]);
+                    rmax = fmax_nan(s_mx[tid + ga.z], s_mx[tid + ga.w]);
                 } else {
                     rmax = -INFINITY;
-                    for (int jb = tid + ga.z; jb <= tid + ga.w; ++jb) rmax = fmaxf(rmax, s_mx[jb]);
+                    for (int jb = tid + ga.z; jb <= tid + ga.w; ++jb) rmax = fmax_nan(rmax, s_mx[jb]);
                 }
                 // prefix bound, with the margin for the rounding of the FP32
                 // prefix; a non-positive bound caps every SNR at 0; NaN stays NaN

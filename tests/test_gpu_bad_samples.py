@@ -39,6 +39,22 @@ def _rows(value, n):
     return x, place.cpu().numpy(), clean
 
 
+def _records(spd, x, msd, widths):
+    """Which samples are records: screened, and every tile."""
+    prm, keep = spd.binding._params(widths, THR, 0, 0, 0)
+    nb = spd.binding.load().spd_detect_workspace_bytes(ctypes.byref(spd.Plane(x).c()),
+                                                       ctypes.byref(prm))
+    for room in (nb, nb - 1):
+        ws = torch.empty(nb, dtype=torch.uint8, device=DEV)[:room]
+        out, res = spd.detect(x, msd, widths, THR, 1 << 20, workspace=ws)
+        count, status = spd.read_result(res)
+        assert status == 0
+        got = np.zeros(x.shape, dtype=bool)
+        rec = spd.candidates_to_numpy(out, count)
+        got[rec["dm"], rec["sample"]] = True
+        yield got
+
+
 def _expected(x, place, msd, widths, starts):
     """Best SNR of each row's starts over the windows inside the row without the sample."""
     y = x.double().cpu().numpy() - msd["mean"][0]
@@ -62,17 +78,7 @@ def _check(spd, value, name, starts, n):
     msd = spd.msd(clean)
     best = _expected(x, place, spd.msd_to_numpy(msd), widths, starts)
     assert (best >= THR).any(axis=1).any()
-    prm, keep = spd.binding._params(widths, THR, 0, 0, 0)
-    nb = spd.binding.load().spd_detect_workspace_bytes(ctypes.byref(spd.Plane(x).c()),
-                                                       ctypes.byref(prm))
-    for room in (nb, nb - 1):      # screened, and every tile
-        ws = torch.empty(nb, dtype=torch.uint8, device=DEV)[:room]
-        out, res = spd.detect(x, msd, widths, THR, 1 << 20, workspace=ws)
-        count, status = spd.read_result(res)
-        assert status == 0
-        got = np.zeros((x.shape[0], n), dtype=bool)
-        rec = spd.candidates_to_numpy(out, count)
-        got[rec["dm"], rec["sample"]] = True
+    for got in _records(spd, x, msd, widths):
         have = np.stack([got[r, place[r] + np.asarray(starts)] for r in range(x.shape[0])])
         sure = np.abs(best - THR) > 1e-3
         assert np.array_equal(have[sure], (best >= THR)[sure])
@@ -91,3 +97,17 @@ def test_starts_before_the_sample(spd, value, name):
 def test_starts_after_the_sample(spd, value, name):
     # every unit after the sample's own, in tiles that are searched whole
     _check(spd, value, name, list(range(16, 64)), 4400)
+
+
+@pytest.mark.parametrize("value", [float("nan"), float("inf"), float("-inf")])
+@pytest.mark.parametrize("n", [2190, 4400])
+def test_starts_after_the_sample_in_its_unit(spd, value, n):
+    """Found by widths to 16; wider ones may miss them."""
+    x, place, clean = _rows(value, n)
+    r = torch.arange(x.shape[0], device=DEV)
+    x[r, torch.from_numpy(place).to(DEV) + 3] = 12.0
+    msd = spd.msd(clean)
+    best = _expected(x, place, spd.msd_to_numpy(msd), list(range(1, 17)), list(range(1, 16)))
+    for got in _records(spd, x, msd, list(range(1, 33))):
+        have = np.stack([got[r, place[r] + np.arange(1, 16)] for r in range(x.shape[0])])
+        assert have[best >= THR + 1e-3].all()
