@@ -1073,7 +1073,8 @@ __device__ __forceinline__ bool search_tiles(const Launch &L, unsigned char *sme
 // of wmax 256) they are searched as units too.  When 15 of 16 tiles are listed,
 // all are searched, as without a screen: in their order in the plane and in
 // chunks, which spares a listed tile its own claim and, with statistics per row,
-// its own load of constants.  1024 x 524288 samples, every tile full of
+// its own load of constants.  (Not where chunks are of one tile anyway: 64 x 65536
+// full of candidates 117 us by the list, 121 without.)  1024 x 524288 samples, every tile full of
 // candidates: 46 widths 7.60 ms by the list and 7.19 so, per row 8.16 and 7.25;
 // widths 1..32 5.71 and 5.20.  With 85 % of the tiles full it is 6.52 and 6.42,
 // per row 7.00 and 6.47, but widths 1..512 (512 x 262144) 6.99 and 7.11.
@@ -1086,7 +1087,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) search_kernel(const __grid_const
         if (L.unit_list) {
             const uint64_t n = *L.tile_count, u = n * (uint32_t)L.units;
             if (u <= 2ull * gridDim.x * (uint32_t)L.live_halves) in_tiles = (uint32_t)u;
-            if (in_tiles || 16 * n < 15 * (uint64_t)L.n_tiles) list = L.tile_list;
+            if (in_tiles || L.chunk == 1 || 16 * n < 15 * (uint64_t)L.n_tiles) list = L.tile_list;
         }
     }
     if (!in_tiles && !search_tiles<DT, G, MG, NT, PL>(L, smem, list)) return;

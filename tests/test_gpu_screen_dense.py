@@ -34,11 +34,12 @@ def _both(spd, x, widths, thr, **kw):
     return got
 
 
-@pytest.mark.parametrize("full", [448, 479, 480, 481, 512])     # of 512 tiles: 14/16 .. 16/16
+# of 5120 tiles (enough for chunks of more than one): 14/16 .. 16/16
+@pytest.mark.parametrize("full", [4480, 4799, 4800, 4801, 5120])
 @pytest.mark.parametrize("scope", [0, 1])
 def test_part_of_the_tiles(spd, full, scope):
     tile = 16 * (256 - ((W46[-1] + 47) // 16 + 1))
-    n_dm, n = 128, 4 * tile
+    n_dm, n = 1280, 4 * tile
     x = synth.noise_plane(n_dm, n, mean=2.0, device=DEV, seed=full)
     g = torch.Generator(device=DEV).manual_seed(full)
     rest = torch.randperm(4 * n_dm, generator=g, device=DEV)[:4 * n_dm - full]
