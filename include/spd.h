@@ -508,8 +508,9 @@ spd_status spd_search_decimated(const spd_plane *plane, const spd_level *levels,
  * extra_bytes > 0 every wait runs out: the kernel sets SPD_ERR_TIMEOUT in the
  * result word and its CTAs leave (each copy itself has landed, so nothing is
  * left in flight).  With 16 every tile is searched; with more the screen stays
- * on, and only listed tiles wait for copies.  spd_debug_set_copy_wait(2000000000, 0) restores the
- * default.  Errors: SPD_ERR_INVALID_ARG. */
+ * on, and only listed tiles wait for copies.
+ * spd_debug_set_copy_wait(2000000000, 0) restores the default.
+ * Errors: SPD_ERR_INVALID_ARG. */
 spd_status spd_debug_set_copy_wait(uint64_t limit_ns, uint32_t extra_bytes);
 
 /* ------------------------------------------------------ de-dispersion

@@ -1074,10 +1074,11 @@ __device__ __forceinline__ bool search_tiles(const Launch &L, unsigned char *sme
 // all are searched, as without a screen: in their order in the plane and in
 // chunks, which spares a listed tile its own claim and, with statistics per row,
 // its own load of constants.  (Not where chunks are of one tile anyway: 64 x 65536
-// full of candidates 117 us by the list, 121 without.)  1024 x 524288 samples, every tile full of
-// candidates: 46 widths 7.60 ms by the list and 7.19 so, per row 8.16 and 7.25;
-// widths 1..32 5.71 and 5.20.  With 85 % of the tiles full it is 6.52 and 6.42,
-// per row 7.00 and 6.47, but widths 1..512 (512 x 262144) 6.99 and 7.11.
+// full of candidates 117 us by the list, 121 without.)  1024 x 524288 samples,
+// every tile full of candidates: 46 widths 7.60 ms by the list and 7.19 so, per
+// row 8.16 and 7.25; widths 1..32 5.71 and 5.20.  With 85 % of the tiles full it
+// is 6.52 and 6.42, per row 7.00 and 6.47, but widths 1..512 (512 x 262144) 6.99
+// and 7.11.
 template <int DT, int G, bool MG, int NT, bool PL>
 __global__ void __launch_bounds__(NT, 512 / NT) search_kernel(const __grid_constant__ Launch L) {
     extern __shared__ __align__(16) unsigned char smem[];
