@@ -6,8 +6,6 @@
 // coupling Sec. 3 names as future work).
 #include "spd_internal.cuh"
 
-#include <type_traits>
-
 namespace spd {
 void note_cuda_error(int e);
 }
@@ -349,16 +347,16 @@ __global__ void __launch_bounds__(kDdThreads, PER == 1 ? 4 : 2) dedisperse_kerne
                 }
             }
         };
-        // a wide spread: channel c straight from global memory, for the first
-        // 4 QUADS trials; the loads of all in flight together
-        auto add_global_to = [&](auto quads, int c) {
+        // a wide spread: channel c straight from global memory, the loads of all
+        // trials in flight together
+        auto add_global = [&](int c) {
             const T *row = fb + (c0 + c) * fb_stride + s_lo[c] + t0 + tid;
             const float sc = has_sc ? __ldg(scale + c0 + c) : 1.f;
             const float of = (has_sc && offset) ? __ldg(offset + c0 + c) : 0.f;
             const int left = (int)min(n_out - t0 - tid, (int64_t)kSpan);   // outputs from the first
             const int4 *dv = reinterpret_cast<const int4 *>(s_dl[c]);
 #pragma unroll
-            for (int q = 0; q < decltype(quads)::value; ++q) {
+            for (int q = 0; q < DMS / 4; ++q) {
                 const int4 d4 = dv[q];   // trials past the block's last read offset 0
                 const int o[4] = {d4.x, d4.y, d4.z, d4.w};
                 T v[4][PER];
@@ -375,16 +373,6 @@ __global__ void __launch_bounds__(kDdThreads, PER == 1 ? 4 : 2) dedisperse_kerne
                         a = __fadd_rn(a, fb_value<DT>(&v[e][j], has_sc, sc, of));
                     }
             }
-        };
-        // a block of few trials reads no others: 128 x 3 x 262144 FP32 with delays
-        // to 1000 pc/cm3 280 us in the middle shape reading 16, 173 so.  (A test
-        // before every four trials keeps their loads from overlapping: 1024 x 16 x
-        // 65536 at the same delays 1.04 ms without, 2.01 with it; in `add`, 216 x
-        // 28 x 48704 172 and 229 us.  The middle shape has no registers to spare.)
-        auto add_global = [&](int c) {
-            if (PER == 4 && nd <= 4) add_global_to(std::integral_constant<int, 1>{}, c);
-            else if (PER == 4 && nd <= 8) add_global_to(std::integral_constant<int, DMS < 8 ? 1 : 2>{}, c);
-            else add_global_to(std::integral_constant<int, DMS / 4>{}, c);
         };
         const uint32_t w0 = (uint32_t)__cvta_generic_to_shared(s_w);
         const uint32_t x0 = (uint32_t)__cvta_generic_to_shared(s_x);
@@ -455,13 +443,17 @@ cudaError_t launch_dd(const spd_plane *fb, const int32_t *delays, int64_t n_dm, 
 // of the middle shape, which form each window for 4 trials only: FP32 48 x 16384
 // (96) 126 in the middle shape and 170 in the small one, 256 x 2000 (64) 112 and
 // 118, 100 x 4000 (56) 117 and 99, 16 x 30000 (59) 140 and 118; FP16 113 and 144 at
-// 64, 122 and 126 at 56.
+// 64, 122 and 126 at 56.  Planes of up to 4 trials that would take the large shape
+// have it in blocks of 4 (one of 16 adds, and where a spread is wide reads, all
+// 16): 128 x 3 x 262144 FP32 147 and 85 us, with delays to 1000 pc/cm3 283 and 140.
 template <int DT>
 cudaError_t launch_dd_dt(const spd_plane *fb, const int32_t *delays, int64_t n_dm, void *out,
                          int out_dt, int64_t n_out, int64_t out_stride, spd_result *status,
                          cudaStream_t s) {
     const int64_t b16 = (n_dm + 15) / 16;
     const int64_t ctas = (n_out + 511) / 512 * b16;
+    if (ctas > 304 && n_dm <= 4)
+        return launch_dd<DT, 4, 4>(fb, delays, n_dm, out, out_dt, n_out, out_stride, status, s);
     if (ctas > 304)
         return launch_dd<DT, 4, 16>(fb, delays, n_dm, out, out_dt, n_out, out_stride, status, s);
     if (ctas >= 64)
